@@ -869,6 +869,11 @@ int launch_rk_small(dg_mesh *m, double *c, double dt, int nsteps, int method, vo
 }
 
 int element_wave(const dg_mesh *m, int *tiles, int *elems_per_tile) {
+  if (m->split_img) {
+    *tiles = split_wave(m);
+    *elems_per_tile = 32;
+    return (int)cudaSuccess;
+  }
 #define CALL(P, NE)                                                                                 \
   (m->rule == DG_RULE_SYMMETRIC                                                                     \
        ? (*elems_per_tile = SfCfg<P, NE, sym_points(P)>::EB, element_sf_per_sm<P, NE, sym_points(P)>(m, tiles)) \
@@ -888,6 +893,7 @@ int element_wave(const dg_mesh *m, int *tiles, int *elems_per_tile) {
 int launch_element(const dg_mesh *m, const double *c, const double *u0, double *out, double *trace_out,
                    const double *fhat, const StageUpdate &su, int mode, void *stream, int64_t e0, int64_t e1) {
   cudaStream_t s = (cudaStream_t)stream;
+  if (m->split_img) return launch_split(m, c, u0, out, trace_out, fhat, su, mode, nullptr, stream, e0, e1);
 #define CALL(P, NE)                                                                                        \
   (m->rule == DG_RULE_SYMMETRIC                                                                            \
        ? run_element_sf<P, NE, sym_points(P)>(m, c, u0, out, trace_out, fhat, su, mode, s, e0, e1)        \

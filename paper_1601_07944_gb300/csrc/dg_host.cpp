@@ -413,6 +413,7 @@ void free_mesh(dg_mesh *m) {
   cudaFree(m->err_flag);
   cudaFree(m->gbar);
   cudaFree(m->tc_img[0]); cudaFree(m->tc_img[1]);
+  cudaFree(m->split_img);
   if (m->copy_stream) cudaStreamDestroy(m->copy_stream);
   for (auto &e : m->copy_ev)
     if (e) cudaEventDestroy(e);
@@ -811,7 +812,8 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       (ce = cudaMemcpy(m->face_geo, fgeo.data(), sizeof(FaceGeo) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->table_block, tb.data(), sizeof(double) * off, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemset(m->err_flag, 0, sizeof(int))) != cudaSuccess ||
-      (ce = (cudaError_t)dg::tc_tables(m)) != cudaSuccess) {
+      (ce = (cudaError_t)dg::tc_tables(m)) != cudaSuccess ||
+      (ce = (cudaError_t)dg::split_tables(m)) != cudaSuccess) {
     free_mesh(m);
     return cuda_fail(ce, "dg_mesh_create: upload");
   }

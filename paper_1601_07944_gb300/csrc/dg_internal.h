@@ -191,6 +191,7 @@ struct dg_mesh {
   dg::GraphCache *graph;
   unsigned *gbar;              // [2] grid barrier of the fused small-mesh stepper (count, generation)
   unsigned char *tc_img[2];    // B operand images of the tensor-core kernel (1xTF32, 3xTF32)
+  unsigned char *split_img;    // table digits of the split-product float64 kernel; null: the mesh does not use it
   int small_stepper;           // dg_set_small_mesh_stepper (on by default)
   cudaStream_t copy_stream;    // dg_rk_step_host's copies out (created on first use)
   cudaEvent_t copy_ev[2];
@@ -241,6 +242,21 @@ int tc_tables_sym(dg_mesh *m);
 int launch_element_tc_sym(const dg_mesh *m, int split3, const double *c, const double *u0, double *out,
                           float *trace_out, const float *fhat, const double *fmean, const StageUpdate &su,
                           int mode, void *stream);
+// The split-product float64 element kernel (dg_split.cuh).  split_tables builds
+// m->split_img (synchronous; at mesh creation) on the meshes that use the kernel:
+// p >= 2 and too many elements for the fused small-mesh stepper, whose results
+// have to be those of the separate launches, bit for bit.  On those meshes
+// launch_element and launch_traces go to launch_split (mode 0/1 as
+// launch_element; mode 2 writes the traces of c, and c to copy when not null).
+int split_tables(dg_mesh *m);
+int split_tables_sym(dg_mesh *m);
+int launch_split(const dg_mesh *m, const double *c, const double *u0, double *out, double *trace_out,
+                 const double *fhat, const StageUpdate &su, int mode, double *copy, void *stream, int64_t e0 = 0,
+                 int64_t e1 = -1);
+int launch_split_sym(const dg_mesh *m, const double *c, const double *u0, double *out, double *trace_out,
+                     const double *fhat, const StageUpdate &su, int mode, double *copy, void *stream, int64_t e0,
+                     int64_t e1);
+int split_wave(const dg_mesh *m);      // tiles (of 32 elements) in flight on the GPU
 int launch_convert_check(int n, unsigned long long *bad, void *stream);
 // The fused small-mesh stepper (float64; the limiter a phase of it when on):
 // nsteps steps of `method` on c in one cooperative launch, the traces of c
