@@ -197,32 +197,25 @@ __device__ __forceinline__ bool lax_friedrichs_edge(const double ul[M], const do
   return positive_finite(ul[0]) & positive_finite(ur[0]) & positive_finite(PL) & positive_finite(PR);
 }
 
-// lax_friedrichs_edge for two float32 traces (an interior face of the mixed
-// modes: the values widen exactly), with two float64 operations fewer per point:
-// one reciprocal serves both sides (1/rho_l = rho_r / (rho_l rho_r), the product
-// of two float32 values being exact in float64), and |rho u|^2 / 2 is formed
-// from the momenta halved in float32 (exact) instead of a multiply by 1/2.
-__device__ __forceinline__ bool lax_friedrichs_edge_f32(const float4 a, const float4 b, const FaceGeo &g,
-                                                        double gamma, double out[M]) {
-  const double g1 = gamma - 1.0;
-  const double ul[M] = {f32_to_f64_dev(a.x), f32_to_f64_dev(a.y), f32_to_f64_dev(a.z), f32_to_f64_dev(a.w)};
-  const double ur[M] = {f32_to_f64_dev(b.x), f32_to_f64_dev(b.y), f32_to_f64_dev(b.z), f32_to_f64_dev(b.w)};
-  const double hxL = f32_to_f64_dev(0.5f * a.y), hyL = f32_to_f64_dev(0.5f * a.z);
-  const double hxR = f32_to_f64_dev(0.5f * b.y), hyR = f32_to_f64_dev(0.5f * b.z);
-  const double ilr = recip(ul[0] * ur[0]);
-  const double il = ur[0] * ilr, ir = ul[0] * ilr;
-  const double wL = fma(ul[1], g.sx, ul[2] * g.sy) * il, wR = fma(ur[1], g.sx, ur[2] * g.sy) * ir;
-  const double PL = fma(-fma(hxL, ul[1], hyL * ul[2]), il, ul[3]);
-  const double PR = fma(-fma(hxR, ur[1], hyR * ur[2]), ir, ur[3]);
-  const double aL = fabs(wL) + sqrt_nr(g.hk * PL * il);
-  const double aR = fabs(wR) + sqrt_nr(g.hk * PR * ir);
-  const double la = max_nonneg(aL, aR);
-  const double wa = wL + la, wb = wR - la, Ps = PL + PR;
-  out[0] = fma(ul[0], wa, ur[0] * wb);
-  out[1] = fma(ul[1], wa, fma(ur[1], wb, Ps * g.gsx));
-  out[2] = fma(ul[2], wa, fma(ur[2], wb, Ps * g.gsy));
-  out[3] = fma(ul[3], wa, fma(ur[3], wb, g1 * fma(PL, wL, PR * wR)));
-  return positive_finite(ul[0]) & positive_finite(ur[0]) & positive_finite(PL) & positive_finite(PR);
+// The same as a call, for the few points that edge_flux_fixed does not take
+// (inlined, its registers would weigh on every point).
+static __device__ __noinline__ bool lax_friedrichs_edge_call(const double *ul, const double *ur, const FaceGeo *g,
+                                                             double gamma, double *out) {
+  return lax_friedrichs_edge(ul, ur, *g, gamma, out);
+}
+
+// l F_hat at one edge point: in fixed point (dg_edgeint.cuh: 10 float64 operations),
+// where the state is out of its range in float64.  False if a side is not physical.
+__device__ __forceinline__ bool edge_flux(const double ul[M], const double ur[M], const FaceFix &ff, const FaceGeo *g,
+                                          double sx, double sy, const GammaFix &gf, double out[M]) {
+  if (edge_flux_fixed(ul, ur, ff, sx, sy, gf.g1, gf.eg, out)) return true;
+  double a[M], b[M], o[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) { a[m] = ul[m]; b[m] = ur[m]; }
+  const bool ok = lax_friedrichs_edge_call(a, b, g, gf.gamma, o);
+#pragma unroll
+  for (int m = 0; m < M; ++m) out[m] = o[m];
+  return ok;
 }
 
 // Ghost state at a point of a boundary face (Algorithm 2: it takes the right
@@ -251,8 +244,9 @@ __device__ __forceinline__ void ghost_state(int code, const double ul[M], double
 template <int NE>
 __device__ __forceinline__ void face_flux_points(const double *__restrict__ trace, double *__restrict__ fhat,
                                                  const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,
-                                                 const double *__restrict__ bstate, int64_t N, int64_t F,
-                                                 double gamma, int *err, int block, int nblocks);
+                                                 const FaceFix *__restrict__ ff, const double *__restrict__ bstate,
+                                                 int64_t N, int64_t F, const GammaFix &gf, int *err, int block,
+                                                 int nblocks);
 
 // device error flag bits (read by dg_device_status)
 constexpr int kErrTimeout = 1;      // a bounded tensor-core wait expired
@@ -278,8 +272,9 @@ __device__ __forceinline__ int64_t checked(int64_t i, int64_t n, int *err) {
 template <int NE>
 __device__ __forceinline__ void face_flux_points(const double *__restrict__ trace, double *__restrict__ fhat,
                                                  const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,
-                                                 const double *__restrict__ bstate, int64_t N, int64_t F,
-                                                 double gamma, int *err, int block, int nblocks) {
+                                                 const FaceFix *__restrict__ ff, const double *__restrict__ bstate,
+                                                 int64_t N, int64_t F, const GammaFix &gf, int *err, int block,
+                                                 int nblocks) {
   constexpr int NF = 3 * NE;
   bool ok = true;
   const int64_t n = F * NE;
@@ -288,14 +283,16 @@ __device__ __forceinline__ void face_flux_points(const double *__restrict__ trac
     const int64_t f = i / NE;
     const int k = (int)(i - f * NE);
     const FaceConn cn = conn[f];
-    const FaceGeo g = fg[f];
+    const FaceGeo *g = fg + f;
+    const FaceFix fix = ff[f];
+    const double sx = g->sx, sy = g->sy;
     const double *pl = trace + ((size_t)checked(cn.l, N, err) * NF + checked(cn.L, 3, err) * NE + k) * M;
     double ul[M], ur[M], Fh[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) ul[m] = pl[m];
     if (cn.r < 0) {
       // boundary face (the first faces of the list): the ghost state at the same point
-      ghost_state(cn.r, ul, g.nx, g.ny, bstate + ((size_t)f * NE + k) * M, ur);
+      ghost_state(cn.r, ul, g->nx, g->ny, bstate + ((size_t)f * NE + k) * M, ur);
     } else {
       const double *pr =
           trace + ((size_t)checked(cn.r, N, err) * NF + checked(cn.R, 3, err) * NE + (NE - 1 - k)) * M;
@@ -303,7 +300,7 @@ __device__ __forceinline__ void face_flux_points(const double *__restrict__ trac
       for (int m = 0; m < M; ++m) ur[m] = pr[m];
     }
     // l * F_hat = (l/2) (F(Ul).n + F(Ur).n - alpha (Ur - Ul))
-    ok &= lax_friedrichs_edge(ul, ur, g, gamma, Fh);
+    ok &= edge_flux(ul, ur, fix, g, sx, sy, gf, Fh);
     double *dst = fhat + (size_t)i * M;
 #pragma unroll
     for (int m = 0; m < M; ++m) dst[m] = Fh[m];

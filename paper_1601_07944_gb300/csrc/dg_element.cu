@@ -736,18 +736,18 @@ template <int P, int NE, int Q, int EBX>
 __global__ void __launch_bounds__(kSmallThreads, 4)
 k_rk_small(double *c, double *S, double *A, double *trace, double *fhat, const double *__restrict__ geo,
            const int32_t *__restrict__ elem_face, const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,
-           const double *__restrict__ bstate, const int32_t *__restrict__ elem_nbr, DevTables tab, int N, int64_t F,
-           double gamma, double phi1, double dt, int nsteps, int method, int limit, unsigned *bar, int *err) {
+           const FaceFix *__restrict__ ff, const double *__restrict__ bstate, const int32_t *__restrict__ elem_nbr, DevTables tab, int N, int64_t F,
+           GammaFix gf, double phi1, double dt, int nsteps, int method, int limit, unsigned *bar, int *err) {
   extern __shared__ double smem[];
   const unsigned nb = gridDim.x;
   const int ns = rk_num_stages(method);
   for (int step = 0; step < nsteps; ++step)
     for (int i = 0; i < ns; ++i) {
       const RkStage st = rk_stage(method, i, dt, c, S, A);
-      face_flux_points<NE>(trace, fhat, conn, fg, bstate, N, F, gamma, err, blockIdx.x, nb);
+      face_flux_points<NE>(trace, fhat, conn, fg, ff, bstate, N, F, gf, err, blockIdx.x, nb);
       if (!grid_barrier(bar, nb, err)) return;
       element_sf_tiles<P, NE, Q, EBX>(smem, st.cin, st.u0, st.out, trace, fhat, geo, elem_face, tab, N, F, st.su, 1,
-                                      gamma, err, blockIdx.x, nb);
+                                      gf.gamma, err, blockIdx.x, nb);
       if (!grid_barrier(bar, nb, err)) return;
       if constexpr (P == 1) {
         // with the limiter on, every stage value is limited in place (and the
@@ -810,17 +810,18 @@ int run_rk_small(dg_mesh *m, double *c, double dt, int nsteps, int method, cudaS
   const int32_t *ef = m->elem_face;
   const FaceConn *conn = m->face_conn;
   const FaceGeo *fg = m->face_geo;
+  const FaceFix *ff = m->face_fix;
   DevTables tab = m->tab;
   int N = (int)m->N;
   int64_t F = m->F;
-  double gamma = m->gamma;
+  GammaFix gf = gamma_fix(m->gamma);
   unsigned *bar = m->gbar;
   int *err = m->err_flag;
   const int32_t *nbr = m->elem_nbr;
   double phi1 = m->phi1;
   int limit = m->limiter ? 1 : 0;
-  void *args[] = {&c,   &S, &A, &tr,    &fh,   &geo, &ef,     &conn,  &fg,   &bst, &nbr, &tab,
-                  &N,   &F, &gamma, &phi1, &dt,   &nsteps, &method, &limit, &bar, &err};
+  void *args[] = {&c,   &S, &A, &tr,    &fh,   &geo, &ef,     &conn,  &fg,   &ff, &bst, &nbr, &tab,
+                  &N,   &F, &gf, &phi1, &dt,   &nsteps, &method, &limit, &bar, &err};
   return (int)cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)nb), dim3(kSmallThreads), args,
                                           Sc::SMEM, s);
 }

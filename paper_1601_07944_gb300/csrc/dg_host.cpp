@@ -406,7 +406,7 @@ bool supported(int p, int ne) {
 void free_mesh(dg_mesh *m) {
   if (!m) return;
   cudaFree(m->geo); cudaFree(m->xy); cudaFree(m->elem_face); cudaFree(m->elem_nbr); cudaFree(m->face_conn);
-  cudaFree(m->face_geo); cudaFree(m->table_block); cudaFree(m->trace); cudaFree(m->fhat);
+  cudaFree(m->face_geo); cudaFree(m->face_fix); cudaFree(m->table_block); cudaFree(m->trace); cudaFree(m->fhat);
   cudaFree(m->stage); cudaFree(m->host_state); cudaFree(m->rk_acc); cudaFree(m->partial); cudaFree(m->totals_dev);
   cudaFree(m->bstate); cudaFree(m->bxy);
   cudaFree(m->adj_buf);
@@ -621,6 +621,8 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       elem_face[3 * f + qf] = 2 * fi + 1;
     }
   const int64_t F = (int64_t)conn.size();
+  std::vector<FaceFix> ffix(F);
+  for (int64_t i = 0; i < F; ++i) ffix[i] = face_fix(fgeo[i].sx, fgeo[i].sy, fgeo[i].hk);
 
   // --- tables ----------------------------------------------------------------
   const int np = (p + 1) * (p + 2) / 2, nd = p + 1, nf = 3 * ne;
@@ -755,6 +757,7 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
   DG_ALLOC(m->elem_nbr, sizeof(int32_t) * N * 3, "element neighbours");
   DG_ALLOC(m->face_conn, sizeof(FaceConn) * F, "face connectivity");
   DG_ALLOC(m->face_geo, sizeof(FaceGeo) * F, "face geometry");
+  DG_ALLOC(m->face_fix, sizeof(FaceFix) * F, "face geometry, fixed point");
   DG_ALLOC(m->table_block, sizeof(double) * off, "tables");
   DG_ALLOC(m->trace, sizeof(double) * N * nf * M, "traces");
   DG_ALLOC(m->fhat, sizeof(double) * F * ne * M, "edge fluxes");
@@ -810,6 +813,7 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       (ce = cudaMemcpy(m->elem_face, elem_face.data(), sizeof(int32_t) * N * 3, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->face_conn, conn.data(), sizeof(FaceConn) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->face_geo, fgeo.data(), sizeof(FaceGeo) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (ce = cudaMemcpy(m->face_fix, ffix.data(), sizeof(FaceFix) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->table_block, tb.data(), sizeof(double) * off, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemset(m->err_flag, 0, sizeof(int))) != cudaSuccess ||
       (ce = (cudaError_t)dg::tc_tables(m)) != cudaSuccess ||

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/dg.h"
+#include "dg_edgeint.cuh"
 
 namespace dg {
 
@@ -30,6 +31,13 @@ struct FaceConn { int32_t l, L, r, R; };
 // (Eq. len); then the products the edge flux uses, formed once on the host with
 // h = l / 2: hk = h^2 gamma (gamma - 1), the scaled normal s = h n, and (gamma - 1) s.
 struct FaceGeo { double nx, ny, hl, hk, sx, sy, gsx, gsy; };
+// gamma, and gamma - 1 in the edge flux's fixed point (edge_flux_fixed)
+struct GammaFix { double gamma; long long g1; int eg; };
+inline GammaFix gamma_fix(double gamma) {
+  const double g1 = gamma - 1.0;
+  const int eg = (int)((fx::bits_of(g1) >> 52) & 0x7FF);
+  return GammaFix{gamma, fx::fixed_of(g1, eg), eg};
+}
 
 struct DevTables {
   // All float64, device.  NP modes, NQ volume points, NF = 3*NE face points.
@@ -167,6 +175,7 @@ struct dg_mesh {
   int32_t *elem_nbr;           // [N][3]: the element across each local face
   dg::FaceConn *face_conn;     // [F]: the Fb boundary faces first (r = boundary code < 0)
   dg::FaceGeo *face_geo;       // [F]
+  dg::FaceFix *face_fix;       // [F] the edge flux's fixed-point geometry
   dg::DevTables tab;
   double *table_block;         // one allocation holding every table
   size_t table_doubles;

@@ -89,9 +89,9 @@ k_traces(const double *__restrict__ c, double *__restrict__ trace, const double 
 template <int NE>
 __global__ void __launch_bounds__(kThreads)
 k_face(const double *__restrict__ trace, double *__restrict__ fhat, const FaceConn *__restrict__ conn,
-       const FaceGeo *__restrict__ fg, const double *__restrict__ bstate, int64_t N, int64_t F, double gamma,
-       int *err) {
-  face_flux_points<NE>(trace, fhat, conn, fg, bstate, N, F, gamma, err, blockIdx.x, gridDim.x);
+       const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff, const double *__restrict__ bstate, int64_t N,
+       int64_t F, GammaFix gf, int *err) {
+  face_flux_points<NE>(trace, fhat, conn, fg, ff, bstate, N, F, gf, err, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -418,7 +418,8 @@ int launch_face_flux(const dg_mesh *m, const double *trace, double *fhat, void *
   do {                                                                                                  \
     static int per_sm = 0;                                                                              \
     k_face<NE><<<resident_grid(m, (const void *)k_face<NE>, kThreads, n, &per_sm), kThreads, 0, s>>>(   \
-        trace, fhat, m->face_conn, m->face_geo, m->bstate, m->N, m->F, m->gamma, m->err_flag);          \
+        trace, fhat, m->face_conn, m->face_geo, m->face_fix, m->bstate, m->N, m->F, gamma_fix(m->gamma),   \
+        m->err_flag);                                                                                   \
   } while (0)
   switch (m->ne) {
     case 2: FACE(2); break;

@@ -32,10 +32,9 @@ namespace {
 
 // Edge flux of the mixed-precision modes, one thread per edge.  The two traces
 // are float32 (exact results of the tensor-core contraction) and are widened
-// exactly; the local Lax-Friedrichs flux is evaluated in float64 at the NE edge
-// points (lax_friedrichs_edge_f32: the flux of k_face, alpha included, with two
-// float64 operations fewer for float32 inputs), with the right element's trace
-// at the reversed point (Eq. edgeint).  Written per
+// exactly; the local Lax-Friedrichs flux is evaluated as in k_face (edge_flux) at
+// the NE edge points, with the right element's trace at the reversed point
+// (Eq. edgeint).  Written per
 // edge: l F_hat at the points rounded to float32 (the lift columns of GEMM 2), and
 // the float64 integral of l F_hat against the constant mode,
 // fmean_m = sum_k omega_k phi_1 l F_hat_{k,m} (Algorithm 2 for j = 1; the
@@ -46,9 +45,9 @@ namespace {
 template <int NE, bool BND>
 __global__ void __launch_bounds__(256)
 k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *__restrict__ fmean,
-             const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const double *__restrict__ Lf,
-             const double *__restrict__ bstate, int np, int64_t N, int64_t f0, int64_t f1, double gamma,
-             int *err) {
+             const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff,
+             const double *__restrict__ Lf, const double *__restrict__ bstate, int np, int64_t N, int64_t f0,
+             int64_t f1, GammaFix gf, int *err) {
   constexpr int NF = 3 * NE;
   bool ok = true;
   // the grid is what is resident at once; block b takes the b-th of gridDim.x
@@ -57,7 +56,9 @@ k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *
   const int64_t lo = f0 + F * blockIdx.x / gridDim.x, hi = f0 + F * (blockIdx.x + 1) / gridDim.x;
   for (int64_t f = lo + threadIdx.x; f < hi; f += blockDim.x) {
     const FaceConn cn = conn[f];
-    const FaceGeo g = fg[f];
+    const FaceGeo *g = fg + f;
+    const FaceFix fix = ff[f];
+    const double sx = g->sx, sy = g->sy;
     // [N][NF][M] float32: one point's four values are one aligned float4
     constexpr bool bnd = BND;
     const int64_t el = checked(cn.l, N, err);
@@ -66,18 +67,21 @@ k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *
                        (bnd ? 0 : checked(cn.R, 3, err) * NE);
     float4 *dst = reinterpret_cast<float4 *>(fhat) + (size_t)f * NE;
     double sm[M] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < NE; ++k) {
       const float4 a = tl[k];
-      double Fh[M];
+      double Fh[M], ur[M];
+      const double ul[M] = {tc::f32_to_f64(a.x), tc::f32_to_f64(a.y), tc::f32_to_f64(a.z), tc::f32_to_f64(a.w)};
       if (bnd) {
-        const double ul[M] = {tc::f32_to_f64(a.x), tc::f32_to_f64(a.y), tc::f32_to_f64(a.z), tc::f32_to_f64(a.w)};
-        double ur[M];
-        ghost_state(cn.r, ul, g.nx, g.ny, bstate + ((size_t)f * NE + k) * M, ur);
-        ok &= lax_friedrichs_edge(ul, ur, g, gamma, Fh);
+        ghost_state(cn.r, ul, g->nx, g->ny, bstate + ((size_t)f * NE + k) * M, ur);
       } else {
-        ok &= lax_friedrichs_edge_f32(a, tr[NE - 1 - k], g, gamma, Fh);
+        const float4 b = tr[NE - 1 - k];
+        ur[0] = tc::f32_to_f64(b.x);
+        ur[1] = tc::f32_to_f64(b.y);
+        ur[2] = tc::f32_to_f64(b.z);
+        ur[3] = tc::f32_to_f64(b.w);
       }
+      ok &= edge_flux(ul, ur, fix, g, sx, sy, gf, Fh);
       const double w = Lf[k * np];           // omega_k phi_1, the same on the three faces
 #pragma unroll
       for (int m = 0; m < M; ++m) sm[m] = fma(w, Fh[m], sm[m]);
@@ -163,13 +167,13 @@ int launch_face_flux_mixed(const dg_mesh *m, const MixedBuffers &b, void *stream
     static int per_sm = 0, per_sm_b = 0;                                                                  \
     k_face_mixed<NE, false><<<resident_grid(m, (const void *)k_face_mixed<NE, false>, 256, m->F - m->Fb,   \
                                             &per_sm), 256, 0, s>>>(                                       \
-        b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->tab.Lf, m->bstate, m->np, m->N, m->Fb, m->F, \
-        m->gamma, m->err_flag);                                                                           \
+        b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N,  \
+        m->Fb, m->F, gamma_fix(m->gamma), m->err_flag);                                                   \
     if (m->Fb > 0)                                                                                        \
       k_face_mixed<NE, true><<<resident_grid(m, (const void *)k_face_mixed<NE, true>, 256, m->Fb,         \
                                              &per_sm_b), 256, 0, s>>>(                                    \
-          b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->tab.Lf, m->bstate, m->np, m->N, 0, m->Fb, \
-          m->gamma, m->err_flag);                                                                         \
+          b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N, \
+          0, m->Fb, gamma_fix(m->gamma), m->err_flag);                                                    \
   } while (0)
   switch (m->ne) {
     case 2: FACE(2); break;

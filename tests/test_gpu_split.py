@@ -141,3 +141,41 @@ def test_non_finite_rows(dgmod, bad):
     near[hit] = True
     near[mesh.nbr[hit]] = True
     assert np.array_equal(got[~near], clean[~near])
+
+
+# The fixed-point edge flux against the oracle's float64 one: still fluid (momenta
+# exactly zero), momenta far below the energies, supersonic flow, jumps inside and
+# beyond the range it takes (a factor of 2^4 between the sides; the float64 form
+# serves the rest), and units in which density and energy are far from one.
+def _gas(rho_pm, p_pm, u, v, scale=1.0):
+    def ic(x, y):
+        s = np.sin(0.7 * x + 0.4 * y)
+        b = np.sign(np.sin(2.1 * x) * np.cos(1.3 * y))
+        return I.primitive_to_conserved(scale * np.exp(rho_pm * b + 0.1 * s), u * (1 + 0.1 * s) + 0.0 * x,
+                                        v * (1 - 0.1 * s) + 0.0 * x, scale * np.exp(p_pm * b - 0.1 * s))
+    return ic
+
+
+@pytest.mark.parametrize("p", [1, 3])
+@pytest.mark.parametrize("ic", [_gas(0, 0, 0, 0), _gas(0, 0, 1e-9, 2e-9), _gas(0.2, 0.1, 9.0, -4.0),
+                                _gas(0.9, 0.9, 0.5, 0.2), _gas(3.0, 4.0, 0.1, 0.3), _gas(0.1, 0.1, 0.7, 0.3, 1e-60),
+                                _gas(0.1, 0.1, 0.7, 0.3, 1e120), _gas(1.0, 0.1, 1e-180, 0.0)],
+                         ids=["rest", "slow", "supersonic", "jumps", "strong_jumps", "tiny_units", "huge_units", "floor"])
+def test_edge_flux_range(dgmod, oracle_mod, p, ic):
+    mesh = I.periodic_mesh(61)
+    m = dgmod.Mesh.from_mesh(mesh, p)
+    o = oracle_mod.OracleDG.from_mesh(mesh, p)
+    cen = mesh.elem_xy.mean(axis=1)
+    c = np.zeros((mesh.n_elem, 4, m.np))
+    c[:, :, 0] = ic(cen[:, 0], cen[:, 1]) / np.sqrt(2.0)          # constant in each element: jumps at every face
+    c[:, :, 1] = 1e-3 * c[:, :, 0]
+    ref, vol = o.rhs_and_volume(c)
+    got = _host(m.rhs(_dev(c)))
+    det = o.det_j()[:, None, None]
+    # the scale of each variable by itself: the edge terms of a piecewise constant
+    # state are as large as h alpha U / det J, which the residual itself shows
+    for k in range(4):
+        scale = np.linalg.norm((vol / det)[:, k]) + np.linalg.norm(ref[:, k])
+        wave = np.linalg.norm(c[:, k] / np.sqrt(det[:, 0])) * 10.0 * max(1.0, np.sqrt(np.max(np.abs(c[:, 3] / c[:, :1, 0][:, 0:1]))))
+        assert np.linalg.norm(got[:, k] - ref[:, k]) <= 1e-12 * scale + 16 * EPS * (scale + wave)
+    m.device_status()
