@@ -129,6 +129,16 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, e, r);
 }
 
+// The same in three float64 operations: with the residual e = 1 - x r of the
+// estimate (|e| < 2^-18), r (1 + e + e^2) leaves e^3 < 2^-54 (checked by
+// dg_self_test alike).
+__device__ __forceinline__ double recip3(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // x > 0 and finite, tested on the bit pattern with integer instructions (a float64
 // compare would take a slot of the narrow float64 pipe)
 __device__ __forceinline__ bool positive_finite(double x) {
@@ -197,6 +207,34 @@ __device__ __forceinline__ bool lax_friedrichs_edge(const double ul[M], const do
   return positive_finite(ul[0]) & positive_finite(ur[0]) & positive_finite(PL) & positive_finite(PR);
 }
 
+// lax_friedrichs_edge for two float32 traces (an interior face of the mixed
+// modes: the values widen exactly), with two float64 operations fewer per point:
+// one reciprocal serves both sides (1/rho_l = rho_r / (rho_l rho_r), the product
+// of two float32 values being exact in float64), and |rho u|^2 / 2 is formed
+// from the momenta halved in float32 (exact) instead of a multiply by 1/2.
+__device__ __forceinline__ bool lax_friedrichs_edge_f32(const float4 a, const float4 b, const FaceGeo &g,
+                                                        double gamma, double out[M]) {
+  const double g1 = gamma - 1.0;
+  const double ul[M] = {f32_to_f64_dev(a.x), f32_to_f64_dev(a.y), f32_to_f64_dev(a.z), f32_to_f64_dev(a.w)};
+  const double ur[M] = {f32_to_f64_dev(b.x), f32_to_f64_dev(b.y), f32_to_f64_dev(b.z), f32_to_f64_dev(b.w)};
+  const double hxL = f32_to_f64_dev(0.5f * a.y), hyL = f32_to_f64_dev(0.5f * a.z);
+  const double hxR = f32_to_f64_dev(0.5f * b.y), hyR = f32_to_f64_dev(0.5f * b.z);
+  const double ilr = recip(ul[0] * ur[0]);
+  const double il = ur[0] * ilr, ir = ul[0] * ilr;
+  const double wL = fma(ul[1], g.sx, ul[2] * g.sy) * il, wR = fma(ur[1], g.sx, ur[2] * g.sy) * ir;
+  const double PL = fma(-fma(hxL, ul[1], hyL * ul[2]), il, ul[3]);
+  const double PR = fma(-fma(hxR, ur[1], hyR * ur[2]), ir, ur[3]);
+  const double aL = fabs(wL) + sqrt_nr(g.hk * PL * il);
+  const double aR = fabs(wR) + sqrt_nr(g.hk * PR * ir);
+  const double la = max_nonneg(aL, aR);
+  const double wa = wL + la, wb = wR - la, Ps = PL + PR;
+  out[0] = fma(ul[0], wa, ur[0] * wb);
+  out[1] = fma(ul[1], wa, fma(ur[1], wb, Ps * g.gsx));
+  out[2] = fma(ul[2], wa, fma(ur[2], wb, Ps * g.gsy));
+  out[3] = fma(ul[3], wa, fma(ur[3], wb, g1 * fma(PL, wL, PR * wR)));
+  return positive_finite(ul[0]) & positive_finite(ur[0]) & positive_finite(PL) & positive_finite(PR);
+}
+
 // The same as a call, for the few points that edge_flux_fixed does not take
 // (inlined, its registers would weigh on every point).
 static __device__ __noinline__ bool lax_friedrichs_edge_call(const double *ul, const double *ur, const FaceGeo *g,
@@ -216,6 +254,17 @@ __device__ __forceinline__ bool edge_flux(const double ul[M], const double ur[M]
 #pragma unroll
   for (int m = 0; m < M; ++m) out[m] = o[m];
   return ok;
+}
+
+static __device__ __noinline__ bool lax_friedrichs_edge_f32_call(float4 a, float4 b, const FaceGeo *g, double gamma,
+                                                                 double *out) {
+  return lax_friedrichs_edge_f32(a, b, *g, gamma, out);
+}
+
+// whether x lies within 512 of its units in the last place of the middle between
+// two float32 values
+__device__ __forceinline__ bool near_f32_tie(double x) {
+  return ((uint32_t)__double2loint(x) & 0x1FFFFFFFu) - (0x10000000u - 512u) < 1024u;
 }
 
 // Ghost state at a point of a boundary face (Algorithm 2: it takes the right

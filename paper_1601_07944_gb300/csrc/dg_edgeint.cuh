@@ -14,6 +14,13 @@
  * mul(a, b) = a b / 2^62, from 31-bit halves.  Both sides share the exponent of
  * the momenta, of the energies and of w, so that sums need no alignment.
  *
+ * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 25 us
+ * (p = 1), 66 -> 34 (p = 2), 87 -> 41 (p = 3), 124 -> 59 (p = 5); k_face_mixed 88 ->
+ * 53 us (p = 3), 403 -> 204 us (512 x 512, p = 4).  About 900 instructions a point,
+ * the integer pipe 53 % busy, the float64 pipe 32 %.  Against 113-bit arithmetic the
+ * error is 0.75-1.0 of the float64 form's (rms) over still, slow, supersonic and
+ * discontinuous states.
+ *
  * A point whose sides differ by more than 2^4 in density or energy, whose state is
  * not physical or not finite, or whose exponents are far from one (beyond 2^300)
  * is left to the float64 form: edge_flux_fixed returns false and writes nothing.
@@ -166,6 +173,19 @@ DG_HD long long recip_mantissa(double x) {
   return ((long long)y << 39) + (z2 >> 13);
 }
 
+// 1/x as a float64, rounded to nearest (to 2^-60 before that).  The sign is x's; a
+// zero, denormal or non-finite x gives NaN, a result below the normal range zero.
+DG_HD double recip_fixed(double x) {
+  const long long b = bits_of(x);
+  const int e = (int)(b >> 52) & 0x7FF;
+  const long long y = recip_mantissa(x);                       // [2^61, 2^62]
+  long long r = ((y + 256) >> 9) + ((long long)(2044 - e) << 52);
+  r = e >= 2045 ? 0 : r;
+  r |= b & (long long)0x8000000000000000ull;
+  r = (unsigned)(e - 1) >= 2046u ? 0x7FF8000000000000ll : r;
+  return of_bits(r);
+}
+
 // sqrt(v) 2^30 for v in [2^58, 2^62): in [2^59, 2^61)
 DG_HD long long sqrt_fixed(long long v) {
   const float f = (float)(int)(v >> 31);                        // v 2^-31, 24 bits
@@ -210,10 +230,11 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   const int em = (int)((mm > (200u << 20) ? mm : (200u << 20)) >> 20);
   const int r0 = rL < rR ? rL : rR, r1 = rL < rR ? rR : rL;
   const int e0 = eL < eR ? eL : eR, eE = eL < eR ? eR : eL;
-  // kinetic energy against total energy: shift of K, exact for a physical state
-  const int dK = eE - 2 * em + r0 - 2;
+  // shift of the kinetic energy K to the scale of E, which keeps six bits free
+  // above it: K of a physical state is below E, but its container may be larger
+  const int dK = eE + 6 - 2 * em + r0 - 2;
   bool ok = (r0 > 723) & (r1 < 1323) & (r1 - r0 <= 4) & (e0 > 723) & (eE < 1323) & (eE - e0 <= 4) & (em < 1323) &
-            (dK >= -6) & (g.es > 0);
+            (dK >= 0) & (g.es > 0);
   if (!ok) return false;
   const Half2x31 Sx = cut(g.sx), Sy = cut(g.sy);
   const Half2x31 G1 = cut(g1);
@@ -232,10 +253,8 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
     w[s] = mul(cut(mn), I);                                     // X = em + es - r0 - 1080
     const long long q = sqr(Mx) + sqr(My);
     const long long K = mul(cut(q), I);                         // |m|^2 / rho, X = 2 em - r0 - 1080
-    const long long Ef = fixed_of(u[3], eE);                    // X = eE - 1083
-    const long long Ks = dK >= 0 ? shr(K, dK) : (long long)((unsigned long long)K << (-dK & 63));
-    Pf[s] = Ef - Ks;                                            // p / (gamma - 1)
-    ok &= Pf[s] > 0 && Ks >= 0 && Ks < (1ll << 62);
+    Pf[s] = (fixed_of(u[3], eE + 6) - shr(K, dK)) * 64;         // p / (gamma - 1), X = eE - 1083
+    ok &= Pf[s] > 0;
     const int z = clz64((unsigned long long)Pf[s]) - 2;         // Pf 2^z in [2^61, 2^62)
     const long long Pn = (long long)((unsigned long long)Pf[s] << (z & 63));
     // c^2 = hk P / rho, h^2 folded in: X = eE - 1083 - z - re + ek + 1

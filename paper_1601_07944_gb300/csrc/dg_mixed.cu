@@ -32,7 +32,7 @@ namespace {
 
 // Edge flux of the mixed-precision modes, one thread per edge.  The two traces
 // are float32 (exact results of the tensor-core contraction) and are widened
-// exactly; the local Lax-Friedrichs flux is evaluated as in k_face (edge_flux) at
+// exactly; the local Lax-Friedrichs flux is evaluated as in k_face (edge_flux_fixed) at
 // the NE edge points, with the right element's trace at the reversed point
 // (Eq. edgeint).  Written per
 // edge: l F_hat at the points rounded to float32 (the lift columns of GEMM 2), and
@@ -43,7 +43,7 @@ namespace {
 // the right, Algorithm 2); otherwise the interior faces [Fb, F), in a separate
 // instantiation so that the common case carries no boundary code.
 template <int NE, bool BND>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *__restrict__ fmean,
              const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff,
              const double *__restrict__ Lf, const double *__restrict__ bstate, int np, int64_t N, int64_t f0,
@@ -81,7 +81,31 @@ k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *
         ur[2] = tc::f32_to_f64(b.z);
         ur[3] = tc::f32_to_f64(b.w);
       }
-      ok &= edge_flux(ul, ur, fix, g, sx, sy, gf, Fh);
+      // The results are rounded to float32 below.  On faces along the axes of a
+      // uniform mesh, between equal traces, they are products of a float32 and a
+      // number of a few bits, and lie in the middle between two float32 values as
+      // often as not: the last float64 bit decides.  Such points take the float64
+      // form, so that the stored flux does not depend on the form of the others.
+      bool done = edge_flux_fixed(ul, ur, fix, sx, sy, gf.g1, gf.eg, Fh);
+      if (done) {
+        bool tie = false;
+#pragma unroll
+        for (int m = 0; m < M; ++m) tie |= near_f32_tie(Fh[m]);
+        done = !tie;
+      }
+      if (!done) {
+        double o[M];
+        if (bnd) {
+          double x[M], y[M];
+#pragma unroll
+          for (int m = 0; m < M; ++m) { x[m] = ul[m]; y[m] = ur[m]; }
+          ok &= lax_friedrichs_edge_call(x, y, g, gf.gamma, o);
+        } else {
+          ok &= lax_friedrichs_edge_f32_call(a, tr[NE - 1 - k], g, gf.gamma, o);
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) Fh[m] = o[m];
+      }
       const double w = Lf[k * np];           // omega_k phi_1, the same on the three faces
 #pragma unroll
       for (int m = 0; m < M; ++m) sm[m] = fma(w, Fh[m], sm[m]);
@@ -122,7 +146,9 @@ __global__ void k_convert_check(int n, unsigned long long *bad) {
   if (ax != 0.0) {
     const long long q = __double_as_longlong(1.0 / ax), r = __double_as_longlong(recip(ax));
     const long long d = q > r ? q - r : r - q;
-    if (d > 1) atomicAdd(bad + 2, 1ull);
+    const long long r3 = __double_as_longlong(recip3(ax)), d3 = q > r3 ? q - r3 : r3 - q;
+    const long long ri = __double_as_longlong(fx::recip_fixed(ax)), di = q > ri ? q - ri : ri - q;
+    if (d > 1 || d3 > 1 || di > 1) atomicAdd(bad + 2, 1ull);
     const long long qs = __double_as_longlong(sqrt(ax)), rs = __double_as_longlong(sqrt_nr(ax));
     const long long ds = qs > rs ? qs - rs : rs - qs;
     const long long qr = __double_as_longlong(1.0 / sqrt(ax)), rr = __double_as_longlong(rsqrt_nr(ax));
