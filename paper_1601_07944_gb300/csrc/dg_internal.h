@@ -253,10 +253,10 @@ int launch_element_tc_sym(const dg_mesh *m, int split3, const double *c, const d
                           int mode, void *stream);
 // The split-product float64 element kernel (dg_split.cuh).  split_tables builds
 // m->split_img (synchronous; at mesh creation) on the meshes that use the kernel:
-// p >= 2 and too many elements for the fused small-mesh stepper, whose results
-// have to be those of the separate launches, bit for bit.  On those meshes
-// launch_element and launch_traces go to launch_split (mode 0/1 as
-// launch_element; mode 2 writes the traces of c, and c to copy when not null).
+// too many elements for the fused small-mesh stepper, whose results have to be
+// those of the separate launches, bit for bit.  On those meshes launch_element and
+// (p >= 2) launch_traces go to launch_split (mode 0/1 as launch_element; mode 2
+// writes the traces of c, and c to copy when not null).
 int split_tables(dg_mesh *m);
 int split_tables_sym(dg_mesh *m);
 int launch_split(const dg_mesh *m, const double *c, const double *u0, double *out, double *trace_out,

@@ -366,7 +366,7 @@ int run_traces(const dg_mesh *m, const double *c, double *trace, double *copy, c
 
 int launch_traces(const dg_mesh *m, const double *c, double *trace, void *stream, double *copy) {
   cudaStream_t s = (cudaStream_t)stream;
-  if (m->split_img)
+  if (m->split_img && m->p > 1)
     return launch_split(m, c, nullptr, nullptr, trace, nullptr, shu_osher(0.0, 0.0, 0.0), 2, copy, stream);
 #define CALL(P, NE) run_traces<P, NE>(m, c, trace, copy, s)
   if (m->p == 1 && m->ne == 2) return CALL(1, 2);

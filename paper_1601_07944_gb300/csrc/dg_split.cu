@@ -7,9 +7,10 @@
 namespace dg {
 
 int split_tables(dg_mesh *m) {
-  if (m->p < 2 || small_rk_fits(m)) return (int)cudaSuccess;
+  if (small_rk_fits(m)) return (int)cudaSuccess;
   if (m->rule == DG_RULE_SYMMETRIC) return split_tables_sym(m);
 #define CALL(P, NE) split_tables_pq<P, NE, 0>(m)
+  if (m->p == 1 && m->ne == 2) return CALL(1, 2);
   if (m->p == 2 && m->ne == 3) return CALL(2, 3);
   if (m->p == 3 && m->ne == 4) return CALL(3, 4);
   if (m->p == 3 && m->ne == 3) return CALL(3, 3);
@@ -26,6 +27,7 @@ int launch_split(const dg_mesh *m, const double *c, const double *u0, double *ou
   if (m->rule == DG_RULE_SYMMETRIC)
     return launch_split_sym(m, c, u0, out, trace_out, fhat, su, mode, copy, stream, e0, e1);
 #define CALL(P, NE) run_split<P, NE, 0>(m, c, u0, out, trace_out, fhat, su, mode, copy, s, e0, e1)
+  if (m->p == 1 && m->ne == 2) return CALL(1, 2);
   if (m->p == 2 && m->ne == 3) return CALL(2, 3);
   if (m->p == 3 && m->ne == 4) return CALL(3, 4);
   if (m->p == 3 && m->ne == 3) return CALL(3, 3);
@@ -35,6 +37,6 @@ int launch_split(const dg_mesh *m, const double *c, const double *u0, double *ou
   return (int)cudaErrorInvalidValue;
 }
 
-int split_wave(const dg_mesh *m) { return m->num_sms * kSplitSubs; }
+int split_wave(const dg_mesh *m) { return m->num_sms * split_groups(m->p); }
 
 }  // namespace dg

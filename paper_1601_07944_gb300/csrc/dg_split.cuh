@@ -25,13 +25,14 @@
  * table entry), rounded once to float64: closer than the float64 sums it
  * replaces, whose every partial sum is rounded to 2^-53.
  *
- * Measured (256 x 256 mesh, 131,072 elements, one launch of a stage, before with
- * k_element_sf -> here): p = 2 0.265 -> 0.174 ms, p = 3 0.498 -> 0.221 ms,
- * p = 4 0.907 -> 0.378 ms, p = 5 1.49 -> 0.515 ms; the symmetric rules 0.242 ->
- * 0.134, 0.593 -> 0.221, 1.08 -> 0.247, 2.07 -> 0.440 ms.  The error of the
- * right-hand side against an 80-bit reference falls by 1.5 (p = 2) to 2.9 (p = 5).
- * Both groups in step, without the turns at the flux (flux_turn): 0.274 ms at
- * p = 3, 0.622 ms at p = 5.
+ * Measured (256 x 256 mesh, 131,072 elements, one launch of a stage, k_element_sf
+ * -> here): p = 1 0.108 -> 0.084 ms, p = 2 0.265 -> 0.128, p = 3 0.498 -> 0.186,
+ * p = 4 0.907 -> 0.327, p = 5 1.49 -> 0.489; the symmetric rules 0.101 -> 0.081,
+ * 0.242 -> 0.115, 0.593 -> 0.172, 1.08 -> 0.225, 2.07 -> 0.403; the traces alone
+ * (mode 2) 0.043 -> 0.033 (p = 2), 0.074 -> 0.041 (p = 3), 0.271 -> 0.072 (p = 5).
+ * The float64 pipe is 60-70 % busy; the rest is the latency of a group's phases,
+ * which the other groups fill only in part.  The error of the right-hand side
+ * against an 80-bit reference falls by 1.5 (p = 2) to 2.9 (p = 5).
  *
  * A row whose largest value is not finite, or is 2^957 or more, gives NaN; values
  * below 2^-959 count as zero.
@@ -39,8 +40,9 @@
  * Layout.  A tile is 32 elements = 128 rows (row = 4 e + m) = 128 TMEM lanes.  A
  * group of 256 threads works on a tile, two threads (halves h = 0, 1) per row:
  * each cuts half of the row's K slots and reassembles half of its outputs.  A CTA
- * holds two groups with barriers of their own that share one copy of the tables,
- * so that one group's integer phases run beside the other's flux phase.  Per tile:
+ * holds three groups (two at p = 5: shared memory) with barriers of their own that
+ * share one copy of the tables, so that one group's integer phases run beside
+ * another's flux phase (split_groups, flux_turn).  Per tile:
  *   GEMM 1  U  = c Phi           interpolation to the volume points
  *           float64 Euler flux, one (element, point) item per thread
  *   GEMM 2  D  = [G_r | G_s | lifted fluxes] [Dr; Ds; Lf]   projection and lift
@@ -65,9 +67,7 @@
 namespace dg {
 namespace {
 
-constexpr int kSplitSubs = 2;                        // tile groups per CTA
-constexpr int kSubThreads = 256;
-constexpr int kSplitThreads = kSplitSubs * kSubThreads;
+constexpr int kSubThreads = 256;                     // threads of a tile group
 constexpr int kDigits = 6;
 constexpr uint64_t kSplitWaitNs = 2000000000ull;     // 2 s per MMA batch before giving up
 constexpr uint32_t kSplitSuspendNs = 1000;
@@ -84,11 +84,19 @@ constexpr int level_cols(int n) {
   return c;
 }
 
+// Tile groups per CTA: three (80 registers a thread, 168 TMEM columns a group, so
+// that GEMM 2 takes its operand in two to five batches) against two (128 registers):
+// p = 2 0.128 against 0.173 ms, p = 3 0.187 against 0.221, p = 4 0.331 against
+// 0.372.  At p = 5 the point buffers of three groups do not fit in shared memory.
+__host__ __device__ constexpr int split_groups(int p) { return p <= 4 ? 3 : 2; }
+
 template <int P, int NE, int Q>
 struct Sp {
   using C = Cfg<P, NE, Q>;
   static constexpr int NP = C::NP, NQ = C::NQ, NF = C::NF;
   static constexpr int EB = 32, ROWS = 128;
+  static constexpr int SUBS = split_groups(P), THREADS = SUBS * kSubThreads;   // tile groups per CTA
+  static constexpr int ROOM = SUBS == 2 ? 256 : 168;        // TMEM columns a group may take
   // outputs and K slots go in halves to a row's two threads
   static constexpr int NPH = half_up(NP), NFH = half_up(NF);
   static constexpr int NB1 = NQ > 16 ? 2 : 1;               // GEMM 1 in batches of points (TMEM columns)
@@ -96,15 +104,15 @@ struct Sp {
   static constexpr int N1 = up8(2 * QH), N2 = up8(2 * NPH), N3 = up8(2 * NFH);
   static constexpr int K1H = up8(NPH), K1 = 2 * K1H;        // GEMMs 1 and 3
   static constexpr int KH = NQ + NFH;                       // GEMM 2: half 0 G_r, half 1 G_s, and half of the fluxes each
-  static constexpr int KROOM = (256 - max2(max2(level_cols(N1), level_cols(N2)), level_cols(N3))) / kDigits / 8 * 8;
+  static constexpr int KROOM = (ROOM - max2(max2(level_cols(N1), level_cols(N2)), level_cols(N3))) / kDigits / 8 * 8;
   static constexpr int NB2 = (up8(KH) + KROOM - 1) / KROOM; // GEMM 2 in batches of K slots
   static constexpr int KC = up8((KH + NB2 - 1) / NB2), K2 = 2 * KC;
   // TMEM columns of a group: the accumulator [0, ND), then the six digit planes
   static constexpr int ND = max2(max2(level_cols(N1), level_cols(N2)), level_cols(N3));
   static constexpr int CA = max2(K1, K2) / 2;
-  static constexpr int SUBCOLS = ND + kDigits * CA <= 128 ? 128 : 256;
-  static_assert(ND + kDigits * CA <= 256, "TMEM columns of a group");
-  static constexpr int COLS = kSplitSubs * SUBCOLS;
+  static constexpr int SUBCOLS = SUBS == 2 ? (ND + kDigits * CA <= 128 ? 128 : 256) : ROOM;
+  static_assert(ND + kDigits * CA <= SUBCOLS, "TMEM columns of a group");
+  static constexpr int COLS = SUBS == 2 ? 2 * SUBCOLS : 512;
   // shared memory: table image (digit blocks, then the three table exponents)
   static constexpr int B1B = kDigits * N1 * K1 * 2, B2B = kDigits * N2 * K2 * 2, B3B = kDigits * N3 * K1 * 2;
   static constexpr int oB1 = 0, oB2 = oB1 + NB1 * B1B, oB3 = oB2 + NB2 * B2B, oEx = oB3 + B3B;
@@ -118,7 +126,7 @@ struct Sp {
   static constexpr int oMx = oG + NG * 32 * 8;              // row exponents: 2 x [2][128], [4][32]
   static constexpr int SUB = oMx + 5 * 128 * 4;
   static constexpr int oSub = (IMG + 127) / 128 * 128;
-  static constexpr int oBar = oSub + kSplitSubs * SUB;      // mbarriers: groups, image; TMEM slot; failure flags
+  static constexpr int oBar = oSub + SUBS * SUB;      // mbarriers: groups, image; TMEM slot; failure flags
   static constexpr int SMEM = oBar + 64;
   static_assert(SMEM <= 227 * 1024, "shared memory");
   static_assert(2 * PT >= ROWS * NP * 8, "mode 2 stages its tile in the point buffers");
@@ -229,14 +237,14 @@ __device__ __forceinline__ double neg_half_bits(double x) {
   return __hiloint2double((__double2hiint(x) ^ (int)0x80000000) - 0x00100000, __double2loint(x));
 }
 
-template <int V>
-struct IntC { static constexpr int value = V; };
-
 // Euler flux of U along two directions a, b (ga, gb = (gamma - 1) times them):
-// 23 float64 operations.  False if the state is not physical.
+// 20 float64 operations (the reciprocal in integers).  False if the state is not physical.
+// FIXED_RECIP: the reciprocal in integers (p >= 4: 0.469 against 0.517 ms at p = 5; at
+// p <= 3, with 80 registers, it costs more than the three float64 operations).
+template <bool FIXED_RECIP>
 __device__ __forceinline__ bool flux_dirs(const double U[M], double ax, double ay, double bx, double by, double gax,
                                           double gay, double gbx, double gby, double g1, double Fa[M], double Fb[M]) {
-  const double inv = recip(U[0]);
+  const double inv = FIXED_RECIP ? fx::recip_fixed(U[0]) : recip3(U[0]);
   const double P = fma(fma(U[1], U[1], U[2] * U[2]), neg_half_bits(inv), U[3]);     // p / (gamma - 1)
   const double Ep = fma(g1, P, U[3]);
   {
@@ -276,11 +284,13 @@ __device__ __forceinline__ void orient_edge_fluxes(uint32_t left, double *f) {
   }
 }
 
-template <int P, int NE, int Q>
-__global__ void __launch_bounds__(kSplitThreads, 1)
+// TRACES: mode 2, in an instantiation of its own (its tile held ahead in registers
+// would weigh on the other modes)
+template <int P, int NE, int Q, bool TRACES>
+__global__ void __launch_bounds__(Sp<P, NE, Q>::THREADS, 1)
 k_element_split(const double *c, const double *u0, double *out, double *__restrict__ trace_out,
                 const double *__restrict__ fhat, const double *__restrict__ geo,
-                const int32_t *__restrict__ elem_face, const unsigned char *__restrict__ img, int N, int64_t F,
+                const int32_t *__restrict__ elem_face, const unsigned char *__restrict__ img, DevTables tab, int N, int64_t F,
                 StageUpdate su, int mode, double gamma, double *__restrict__ copy, int *err) {
   using T = Sp<P, NE, Q>;
   constexpr int NP = T::NP, NQ = T::NQ, NF = T::NF, EB = T::EB, LD = T::LD, NPH = T::NPH, NFH = T::NFH;
@@ -297,16 +307,16 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
   uint32_t *sMxB = sMxA + 256;                               // the same, for the new state
   uint32_t *sMxG = sMxB + 256;                               // [4][32] largest high word of the flux rows
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm + T::oBar);
-  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + T::oBar + 32);
+  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + T::oBar + 36);
   volatile int *fail = reinterpret_cast<volatile int *>(sm + T::oBar + 48);
   int *turn = reinterpret_cast<int *>(sm + T::oBar + 40);
-  const uint32_t mbar = tc::smem_u32(bars + sub), mbar_img = tc::smem_u32(bars + kSplitSubs);
+  const uint32_t mbar = tc::smem_u32(bars + sub), mbar_img = tc::smem_u32(bars + T::SUBS);
 
   // ---- once per CTA: TMEM, mbarriers, the table image ----
   if (threadIdx.x < 32) tc::tmem_alloc(tc::smem_u32(slot), T::COLS);
   if (threadIdx.x == 0) {
-    for (int i = 0; i <= kSplitSubs; ++i) tc::mbar_init(tc::smem_u32(bars + i), 1);
-    for (int i = 0; i < kSplitSubs; ++i) fail[i] = 0;
+    for (int i = 0; i <= T::SUBS; ++i) tc::mbar_init(tc::smem_u32(bars + i), 1);
+    for (int i = 0; i < T::SUBS; ++i) fail[i] = 0;
     *turn = 0;
   }
   tc::fence_proxy_async();
@@ -320,8 +330,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
   }
   const bool img_ok = tc::mbar_wait_sleep(mbar_img, 0, kSplitWaitNs, kSplitSuspendNs);
   if (!img_ok) {
-    fail[0] = 1;
-    fail[1] = 1;
+    for (int i = 0; i < T::SUBS; ++i) fail[i] = 1;
     atomicOr(err, kErrTimeout);
   }
   __syncthreads();
@@ -356,13 +365,14 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
   // the larger of the two halves' values (a barrier of the row's two warps)
   auto pair_max = [&](uint32_t *s, uint32_t v) -> uint32_t {
     s[h * 128 + row] = v;
-    bar_sync(1 + kSplitSubs + sub * 4 + quarter, 64);
+    bar_sync(1 + T::SUBS + sub * 4 + quarter, 64);
     return max(v, s[(h ^ 1) * 128 + row]);
   };
   // One group of the CTA in the flux phase at a time: the float64 pipe serves one
   // group as fast as two, and taking turns keeps the groups out of step, so that
-  // one's integer phases run beside the other's flux.  A wait that does not end
-  // soon goes ahead (the order is for speed only).
+  // one's integer phases run beside another's flux (two groups, p = 3: 0.221 against
+  // 0.274 ms without turns; three groups: 0.202, two of them at once 0.214).  A wait
+  // that does not end soon goes ahead (the order is for speed only).
   auto flux_turn = [&]() {
     if (tid != 0) return;
     for (int i = 0; i < 400; ++i) {
@@ -383,26 +393,40 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
 
   const int ntiles = (N + EB - 1) / EB;
   const bool need_u0 = mode == 1 && su.a0 != 0.0;
-  // a tile's inputs, loaded ahead of it: this half's modes (p <= 3: further up the
-  // registers do not reach), the element's edges, and (a component per warp, the
-  // element across the lanes) the geometry
-  constexpr bool AHEAD = P <= 3;
-  double cn[AHEAD ? NPH : 1], geo_n = 0.0;
-  int ef[3] = {0, 0, 0};
   auto load_modes = [&](int tile, double *v) {
     const int e0 = tile * EB;
-    const bool on = tile < ntiles && e0 + rel < N;
+    const bool on = e0 + rel < N;
     const size_t o = ((size_t)(e0 + rel) * M + rm) * NP + h * NPH;
 #pragma unroll
     for (int i = 0; i < NPH; ++i) v[i] = on && h * NPH + i < NP ? c[o + i] : 0.0;
   };
+  // With three groups (80 registers a thread) the edge fluxes are loaded beside the
+  // flux of the points and the modes once more for the update; with two, both at the
+  // start of the tile (p = 5: 0.476 against 0.502 ms; p = 3: 0.187 against 0.193).
+  constexpr bool LATE = T::SUBS == 3;
+  // a tile's edges and (a component per warp, the element across the lanes)
+  // geometry, loaded ahead of it
+  double geo_n = 0.0;
+  int ef[3] = {0, 0, 0};
+  auto edge_fluxes = [&](double *fl, bool live) {
+    if (h == 0) load_edge_fluxes<NE, NFH, 0>(fhat, ef, rm, live, F, err, fl);
+    else load_edge_fluxes<NE, NFH, 1>(fhat, ef, rm, live, F, err, fl);
+  };
   auto load_inputs = [&](int tile) {
     const int e0 = tile * EB;
     const bool on = tile < ntiles && e0 + rel < N;
-    if constexpr (AHEAD) load_modes(tile, cn);
 #pragma unroll
     for (int q = 0; q < 3; ++q) ef[q] = on ? elem_face[(size_t)(e0 + rel) * 3 + q] : 0;
     geo_n = warp < 5 && tile < ntiles && e0 + lane < N ? geo[(size_t)(e0 + lane) * GEO + warp] : 0.0;
+  };
+  constexpr int TV = (EB * M * NP + kSubThreads - 1) / kSubThreads;
+  double tv[TRACES ? TV : 1];
+  auto load_tile = [&](int tile) {
+#pragma unroll
+    for (int x = 0; x < TV; ++x) {
+      const int i = tid + x * kSubThreads;
+      tv[x] = tile < ntiles && i < min(EB, N - tile * EB) * M * NP ? c[(size_t)tile * EB * M * NP + i] : 0.0;
+    }
   };
   auto tile_body = [&](int tile, int next) -> bool {
     const int e0 = tile * EB, ecount = min(EB, N - e0);
@@ -410,31 +434,24 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
     const size_t orow = ((size_t)(e0 + rel) * M + rm) * NP;
     double cv[NPH], fl[NFH];
     uint32_t left = 0u;                                      // bit q: this is edge q's left element
-    if (mode == 2) {
-      // the tile through shared memory, whole rows of it in order (c may be host memory)
-      for (int i = tid; i < EB * M * NP; i += kSubThreads) {
-        double v = 0.0;
-        if (i < ecount * M * NP) {
-          v = c[(size_t)e0 * M * NP + i];
-          if (copy) copy[(size_t)e0 * M * NP + i] = v;
-        }
-        sU[i] = v;
+    if constexpr (TRACES) {
+      // the tile through shared memory, whole rows of it in order (c may be host
+      // memory), loaded a tile ahead
+#pragma unroll
+      for (int x = 0; x < TV; ++x) {
+        const int i = tid + x * kSubThreads;
+        if (copy && i < ecount * M * NP) copy[(size_t)e0 * M * NP + i] = tv[x];
+        if (i < EB * M * NP) sU[i] = tv[x];
       }
       if (!sub_sync()) return false;
+      load_tile(next);
 #pragma unroll
       for (int i = 0; i < NPH; ++i) cv[i] = h * NPH + i < NP ? sU[row * NP + h * NPH + i] : 0.0;
     } else {
-      // (the edge fluxes stay in flight until GEMM 1 is done)
-      if (h == 0) load_edge_fluxes<NE, NFH, 0>(fhat, ef, rm, live, F, err, fl);
-      else load_edge_fluxes<NE, NFH, 1>(fhat, ef, rm, live, F, err, fl);
+      if constexpr (!LATE) edge_fluxes(fl, live);
 #pragma unroll
       for (int q = 0; q < 3; ++q) left |= (ef[q] & 1) ? 0u : 1u << q;
-      if constexpr (AHEAD) {
-#pragma unroll
-        for (int i = 0; i < NPH; ++i) cv[i] = cn[i];
-      } else {
-        load_modes(tile, cv);
-      }
+      load_modes(tile, cv);
     }
     uint32_t mx = 0;
 #pragma unroll
@@ -442,7 +459,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
     mx = pair_max(sMxA, mx);
     int E = row_exp(mx);
     uint32_t nan = mx >= (1980u << 20) ? 0x7FF80000u : 0u;
-    if (mode != 2) {
+    if constexpr (!TRACES) {
       store_modes(cv, E);
       if (warp < 4) {
         sGeo[warp * 32 + lane] = geo_n;
@@ -483,38 +500,27 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       }
       // ---- float64 flux, one point per warp and turn, the element across the lanes ----
       {
+        if constexpr (LATE) edge_fluxes(fl, live);
         bool phys = true;
         uint32_t gm[M] = {0u, 0u, 0u, 0u};
         double g[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) g[i] = sGeo[i * 32 + lane];
-        constexpr int W = kSubThreads / 32;
-        auto points = [&](auto ni, int k0) {                 // points k0, k0 + W, ... at once
-          constexpr int NI = decltype(ni)::value;
-          double U[NI][M], Gr[NI][M], Gs[NI][M];
+        for (int k = warp; k < NQ; k += kSubThreads / 32) {
+          double *pu = sU + k * M * LD + lane, *ps = sS + k * M * LD + lane;
+          double U[M], Gr[M], Gs[M];
 #pragma unroll
-          for (int x = 0; x < NI; ++x)
+          for (int m = 0; m < M; ++m) U[m] = pu[m * LD];
+          phys &= flux_dirs<(P >= 4)>(U, g[0], g[1], g[2], g[3], g[4], g[5], g[6], g[7], g1, Gr, Gs) || lane >= ecount;
 #pragma unroll
-            for (int m = 0; m < M; ++m) U[x][m] = sU[((k0 + x * W) * M + m) * LD + lane];
-#pragma unroll
-          for (int x = 0; x < NI; ++x) {
-            const bool ok = flux_dirs(U[x], g[0], g[1], g[2], g[3], g[4], g[5], g[6], g[7], g1, Gr[x], Gs[x]);
-            phys &= ok || lane >= ecount;
+          for (int m = 0; m < M; ++m) {
+            if (lane >= ecount) { Gr[m] = 0.0; Gs[m] = 0.0; }
+            pu[m * LD] = Gr[m];
+            ps[m * LD] = Gs[m];
+            gm[m] = max(gm[m], max((uint32_t)__double2hiint(Gr[m]) & 0x7FFFFFFFu,
+                                   (uint32_t)__double2hiint(Gs[m]) & 0x7FFFFFFFu));
           }
-#pragma unroll
-          for (int x = 0; x < NI; ++x)
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-              if (lane >= ecount) { Gr[x][m] = 0.0; Gs[x][m] = 0.0; }
-              sU[((k0 + x * W) * M + m) * LD + lane] = Gr[x][m];
-              sS[((k0 + x * W) * M + m) * LD + lane] = Gs[x][m];
-              gm[m] = max(gm[m], max((uint32_t)__double2hiint(Gr[x][m]) & 0x7FFFFFFFu,
-                                     (uint32_t)__double2hiint(Gs[x][m]) & 0x7FFFFFFFu));
-            }
-        };
-        int k = warp;
-        for (; k + W < NQ; k += 2 * W) points(IntC<2>{}, k);
-        if (k < NQ) points(IntC<1>{}, k);
+        }
         if (!phys) atomicOr(err, kErrNonPhysical);
 #pragma unroll
         for (int m = 0; m < M; ++m) atomicMax(&sMxG[m * 32 + lane], gm[m]);
@@ -554,6 +560,8 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       }
 #pragma unroll
       for (int i = 0; i < NPH; ++i) uv[i] = need_u0 && live && h * NPH + i < NP ? u0[orow + h * NPH + i] : 0.0;
+      if constexpr (LATE)
+        if (mode != 0) load_modes(tile, cv);
       mma_wait();
       // ---- stage update ----
       {
@@ -574,8 +582,11 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
                 v = D * kap;
               } else {
                 // a0 u0 + b0 c + g dt R with R = D / det J
-                double t = su.b0 == 1.0 ? cv[jj < NPH ? jj : 0] : su.b0 * cv[jj < NPH ? jj : 0];
-                if (need_u0) t = fma(su.a0, uv[jj < NPH ? jj : 0], t);
+                const double cj = cv[jj < NPH ? jj : 0], uj = uv[jj < NPH ? jj : 0];
+                double t;
+                if (su.b0 == 0.0) t = su.a0 == 1.0 ? uj : su.a0 * uj;
+                else t = su.b0 == 1.0 ? cj : su.b0 * cj;
+                if (need_u0 && su.b0 != 0.0) t = fma(su.a0, uj, t);
                 v = fma(kap, D, t);
                 if (su.out2 && live) {
                   double t2 = su.y * v;
@@ -591,6 +602,28 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
         tc::fence_before_sync();
       }
       load_inputs(next);
+      if constexpr (P == 1) {
+        // p = 1: the edge traces in float64, by the sums of every other kernel that
+        // writes traces (the limiter recomputes those of limited elements)
+        if (trace_out) {
+          double *sN = sU + row * NP + h * NPH;
+#pragma unroll
+          for (int i = 0; i < NPH; ++i)
+            if (h * NPH + i < NP) sN[i] = cv[i];
+          if (!sub_sync()) return false;
+          const double *cj = sU + row * NP;
+          double z[P + 2], t0, t1, t2;
+          face_sums<P>(cj, tab.EChiM1, tab.EChi[0], z);
+          edge_traces_unit<P, NE>(cj, z, tab.EPa, tab.EChi, h, t0, t1, t2);
+          if (live) {
+            double *dst = trace_out + (size_t)(e0 + rel) * NF * M + rm;
+            dst[h * M] = t0;
+            dst[(NE + h) * M] = t1;
+            dst[(3 * NE - 1 - h) * M] = t2;
+          }
+        }
+        return sub_sync();
+      }
       if (!trace_out) return sub_sync();       // the next tile overwrites the geometry read above
       // ---- the new state's row exponents ----
       mx = 0;
@@ -629,8 +662,9 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
   };
 
   bool ok = img_ok && fail[sub] == 0;
-  const int first = sub * (int)gridDim.x + (int)blockIdx.x, step = kSplitSubs * (int)gridDim.x;
-  if (mode != 2) load_inputs(first);
+  const int first = sub * (int)gridDim.x + (int)blockIdx.x, step = T::SUBS * (int)gridDim.x;
+  if constexpr (TRACES) load_tile(first);
+  else load_inputs(first);
   for (int tile = first; ok && tile < ntiles; tile += step) ok = tile_body(tile, tile + step);
   // a wait expired: wait (bounded again) for that batch, so that no MMA writes the
   // columns freed below, and for the image's copy
@@ -738,8 +772,10 @@ int run_split(const dg_mesh *m, const double *c, const double *u0, double *out, 
               const StageUpdate &su0, int mode, double *copy, cudaStream_t s, int64_t e0, int64_t e1) {
   using T = Sp<P, NE, Q>;
   static PerDevice attr_set;
+  auto stage = k_element_split<P, NE, Q, false>, traces = k_element_split<P, NE, Q, (P > 1)>;   // p = 1: k_traces
   if (!attr_set.test(m->device)) {
-    cudaError_t e = cudaFuncSetAttribute(k_element_split<P, NE, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(stage, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(traces, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
     if (e != cudaSuccess) return (int)e;
     attr_set.set(m->device);
   }
@@ -752,10 +788,10 @@ int run_split(const dg_mesh *m, const double *c, const double *u0, double *out, 
   if (su.out2) su.out2 += so;
   const int64_t ntiles = (n + T::EB - 1) / T::EB;
   const int grid = (int)(ntiles < m->num_sms ? ntiles : m->num_sms);
-  k_element_split<P, NE, Q><<<grid, kSplitThreads, T::SMEM, s>>>(
+  (mode == 2 ? traces : stage)<<<grid, T::THREADS, T::SMEM, s>>>(
       c + so, u0 ? u0 + so : nullptr, out ? out + so : nullptr,
       trace_out ? trace_out + (size_t)e0 * T::NF * M : nullptr, fhat, m->geo + (size_t)e0 * GEO,
-      m->elem_face + (size_t)e0 * 3, m->split_img, (int)n, m->F, su, mode, m->gamma, copy ? copy + so : nullptr,
+      m->elem_face + (size_t)e0 * 3, m->split_img, m->tab, (int)n, m->F, su, mode, m->gamma, copy ? copy + so : nullptr,
       m->err_flag);
   return (int)cudaGetLastError();
 }

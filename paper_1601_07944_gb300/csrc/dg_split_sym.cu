@@ -8,6 +8,7 @@ namespace dg {
 
 int split_tables_sym(dg_mesh *m) {
 #define CALL(P, NE) split_tables_pq<P, NE, sym_points(P)>(m)
+  if (m->p == 1 && m->ne == 2) return CALL(1, 2);
   if (m->p == 2 && m->ne == 3) return CALL(2, 3);
   if (m->p == 3 && m->ne == 4) return CALL(3, 4);
   if (m->p == 3 && m->ne == 3) return CALL(3, 3);
@@ -22,6 +23,7 @@ int launch_split_sym(const dg_mesh *m, const double *c, const double *u0, double
                      int64_t e1) {
   cudaStream_t s = (cudaStream_t)stream;
 #define CALL(P, NE) run_split<P, NE, sym_points(P)>(m, c, u0, out, trace_out, fhat, su, mode, copy, s, e0, e1)
+  if (m->p == 1 && m->ne == 2) return CALL(1, 2);
   if (m->p == 2 && m->ne == 3) return CALL(2, 3);
   if (m->p == 3 && m->ne == 4) return CALL(3, 4);
   if (m->p == 3 && m->ne == 3) return CALL(3, 3);
