@@ -121,67 +121,70 @@ __device__ __forceinline__ int mode_a_ge1(int r) {
   return d * (d + 1) / 2 + (r - d * (d - 1) / 2);
 }
 
-// The element stage on the tiles block, block + nblocks, ... (k_element_sf, and
-// the element phase of the fused small-mesh stepper); smem holds SfCfg::SMEM bytes.
+// One tile of the element stage in shared memory (SfCfg::SMEM bytes), in phases that
+// the element kernel and the fused small-mesh stepper put together in different
+// orders; each phase leaves the synchronisation before the next to its caller
+// unless it says otherwise.
 template <int P, int NE, int Q, int EBX = 0>
-__device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, const double *u0, double *out,
-                                                 double *__restrict__ trace_out, const double *__restrict__ fhat,
-                                                 const double *__restrict__ geo, const int32_t *__restrict__ elem_face,
-                                                 const DevTables &tab, int N, int64_t F, const StageUpdate &su,
-                                                 int mode, double gamma, int *err, int block, int nblocks) {
+struct SfTile {
   using S = SfCfg<P, NE, Q, EBX>;
-  constexpr int NP = S::NP, ND = S::ND, NQ = S::NQ, NF = S::NF, EB = S::EB;
-  double *sPa = smem;                  // [ND][ND]   P_a(alpha_ia)
-  double *sPaW = sPa + ND * ND;        // [ND][ND]   wa P_a
-  double *sdPaW = sPaW + ND * ND;      // [ND][ND]   wa P_a'
-  double *sChi = sdPaW + ND * ND;      // [NP][ND]   chi_j(beta_ib)
-  double *sChiA = sChi + NP * ND;      // [NP][ND]   chi_j wb / (4 (1-s))
-  double *sdChiB = sChiA + NP * ND;    // [NP][ND]   chi_j' wb / 4
-  double *sHalf = sdChiB + NP * ND;    // [ND]       (1 + alpha_ia) / 2
-  double *sEChi = sHalf + ND;          // [NP][NE]   chi_j(xi_k)
-  double *sEWChi = sEChi + NP * NE;    // [NP][NE]   omega_k chi_j(xi_k)
-  double *sEWPa = sEWChi + NP * NE;    // [ND][NE]   omega_k P_a(xi_k)
-  double *sEChiM1 = sEWPa + ND * NE;   // [NP]       chi_j(-1)
-  double *sEPa = sEChiM1 + NP;         // [ND][NE]   P_a(xi_k)
-  double *sBvT = sEPa + ND * NE;       // direct form: [NP][NQ] phi_j(r_k)
-  double *sDr = sBvT + (S::DIRECT ? NP * NQ : 0);   //  [NQ][NP] w_k d_r phi_j(r_k)
-  double *sDs = sDr + (S::DIRECT ? NQ * NP : 0);    //  [NQ][NP] w_k d_s phi_j(r_k)
-  double *sC = sDs + (S::DIRECT ? NQ * NP : 0);     // [EB][M][NP]        stage input
-  double *sX = sC + EB * M * NP;       // [EB][ND][ND][8]    W (first 4), then Xa, Xb (direct: the new state)
-  double *sH = sX + EB * S::XS;        // [EB][NQ][8]        Ha, Hb (direct: G_r, G_s); later the new state
-  double *sF = sH + EB * NQ * 8;       // [EB][RS][M]        -F_hat_out * l, then the lift sums
-  double *sDir = sF + EB * S::RS * M;  // [EB][ND+1][2]      J^tau row 0 + half_ia row 1 (ia < ND), row 1
-  double *sO = S::DIRECT ? sX : sH;
-  constexpr int RS = S::RS;
+  static constexpr int NP = S::NP, ND = S::ND, NQ = S::NQ, NF = S::NF, EB = S::EB, RS = S::RS;
+  double *sPa, *sPaW, *sdPaW, *sChi, *sChiA, *sdChiB, *sHalf, *sEChi, *sEWChi, *sEWPa, *sEChiM1, *sEPa;
+  double *sBvT, *sDr, *sDs, *sC, *sX, *sH, *sF, *sDir, *sO;
 
-  for (int i = threadIdx.x; i < ND * ND; i += blockDim.x) {
-    sPa[i] = tab.SPa[i]; sPaW[i] = tab.SPaW[i]; sdPaW[i] = tab.SdPaW[i];
+  __device__ __forceinline__ explicit SfTile(double *smem) {
+    sPa = smem;                  // [ND][ND]   P_a(alpha_ia)
+    sPaW = sPa + ND * ND;        // [ND][ND]   wa P_a
+    sdPaW = sPaW + ND * ND;      // [ND][ND]   wa P_a'
+    sChi = sdPaW + ND * ND;      // [NP][ND]   chi_j(beta_ib)
+    sChiA = sChi + NP * ND;      // [NP][ND]   chi_j wb / (4 (1-s))
+    sdChiB = sChiA + NP * ND;    // [NP][ND]   chi_j' wb / 4
+    sHalf = sdChiB + NP * ND;    // [ND]       (1 + alpha_ia) / 2
+    sEChi = sHalf + ND;          // [NP][NE]   chi_j(xi_k)
+    sEWChi = sEChi + NP * NE;    // [NP][NE]   omega_k chi_j(xi_k)
+    sEWPa = sEWChi + NP * NE;    // [ND][NE]   omega_k P_a(xi_k)
+    sEChiM1 = sEWPa + ND * NE;   // [NP]       chi_j(-1)
+    sEPa = sEChiM1 + NP;         // [ND][NE]   P_a(xi_k)
+    sBvT = sEPa + ND * NE;       // direct form: [NP][NQ] phi_j(r_k)
+    sDr = sBvT + (S::DIRECT ? NP * NQ : 0);   //  [NQ][NP] w_k d_r phi_j(r_k)
+    sDs = sDr + (S::DIRECT ? NQ * NP : 0);    //  [NQ][NP] w_k d_s phi_j(r_k)
+    sC = sDs + (S::DIRECT ? NQ * NP : 0);     // [EB][M][NP]        stage input
+    sX = sC + EB * M * NP;       // [EB][ND][ND][8]    W (first 4), then Xa, Xb (direct: the new state)
+    sH = sX + EB * S::XS;        // [EB][NQ][8]        Ha, Hb (direct: G_r, G_s); later the new state
+    sF = sH + EB * NQ * 8;       // [EB][RS][M]        -F_hat_out * l, then the lift sums
+    sDir = sF + EB * RS * M;     // [EB][ND+1][2]      J^tau row 0 + half_ia row 1 (ia < ND), row 1
+    sO = S::DIRECT ? sX : sH;    // the new state
   }
-  for (int i = threadIdx.x; i < NP * ND; i += blockDim.x) {
-    sChi[i] = tab.SChi[i]; sChiA[i] = tab.SChiA[i]; sdChiB[i] = tab.SdChiB[i];
-  }
-  for (int i = threadIdx.x; i < ND; i += blockDim.x) sHalf[i] = tab.SHalf[i];
-  for (int i = threadIdx.x; i < NP * NE; i += blockDim.x) { sEChi[i] = tab.EChi[i]; sEWChi[i] = tab.EWChi[i]; }
-  for (int i = threadIdx.x; i < ND * NE; i += blockDim.x) sEWPa[i] = tab.EWPa[i];
-  for (int i = threadIdx.x; i < NP; i += blockDim.x) sEChiM1[i] = tab.EChiM1[i];
-  for (int i = threadIdx.x; i < ND * NE; i += blockDim.x) sEPa[i] = tab.EPa[i];
-  if constexpr (S::DIRECT) {
-    for (int i = threadIdx.x; i < NP * NQ; i += blockDim.x) {
-      sBvT[i] = tab.BvT[i]; sDr[i] = tab.Dr[i]; sDs[i] = tab.Ds[i];
+
+  __device__ __forceinline__ void load_tables(const DevTables &tab) {
+    for (int i = threadIdx.x; i < ND * ND; i += blockDim.x) {
+      sPa[i] = tab.SPa[i]; sPaW[i] = tab.SPaW[i]; sdPaW[i] = tab.SdPaW[i];
+    }
+    for (int i = threadIdx.x; i < NP * ND; i += blockDim.x) {
+      sChi[i] = tab.SChi[i]; sChiA[i] = tab.SChiA[i]; sdChiB[i] = tab.SdChiB[i];
+    }
+    for (int i = threadIdx.x; i < ND; i += blockDim.x) sHalf[i] = tab.SHalf[i];
+    for (int i = threadIdx.x; i < NP * NE; i += blockDim.x) { sEChi[i] = tab.EChi[i]; sEWChi[i] = tab.EWChi[i]; }
+    for (int i = threadIdx.x; i < ND * NE; i += blockDim.x) sEWPa[i] = tab.EWPa[i];
+    for (int i = threadIdx.x; i < NP; i += blockDim.x) sEChiM1[i] = tab.EChiM1[i];
+    for (int i = threadIdx.x; i < ND * NE; i += blockDim.x) sEPa[i] = tab.EPa[i];
+    if constexpr (S::DIRECT) {
+      for (int i = threadIdx.x; i < NP * NQ; i += blockDim.x) {
+        sBvT[i] = tab.BvT[i]; sDr[i] = tab.Dr[i]; sDs[i] = tab.Ds[i];
+      }
     }
   }
 
-  const int ntiles = (N + EB - 1) / EB;
-  for (int tile = block; tile < ntiles; tile += nblocks) {
-    const int e0 = tile * EB;
-    const int ecount = min(EB, N - e0);
-    __syncthreads();
+  // the stage input
+  __device__ __forceinline__ void load_state(const double *c, int e0, int ecount) {
     const double *src = c + (size_t)e0 * M * NP;
-    for (int i = threadIdx.x; i < EB * M * NP; i += blockDim.x)
-      sC[i] = i < ecount * M * NP ? src[i] : 0.0;
+    for (int i = threadIdx.x; i < EB * M * NP; i += blockDim.x) sC[i] = i < ecount * M * NP ? src[i] : 0.0;
+  }
+
+  // the flux is linear in its direction: H_alpha = G_r + half G_s is the flux
+  // along J^tau row 0 + half row 1, H_beta = G_s the flux along row 1
+  __device__ __forceinline__ void load_dirs(const double *__restrict__ geo, int e0, int ecount) {
     if constexpr (S::PREDIR) {
-      // the flux is linear in its direction: H_alpha = G_r + half G_s is the flux
-      // along J^tau row 0 + half row 1, H_beta = G_s the flux along row 1
       for (int i = threadIdx.x; i < EB * (ND + 1); i += blockDim.x) {
         const int el = i / (ND + 1), ia = i - el * (ND + 1);
         double dx = 0.0, dy = 0.0;
@@ -200,12 +203,17 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
         sDir[2 * i + 1] = dy;
       }
     }
+  }
+
+  // the element's edge fluxes in its own order, -F_hat_out l; edge(el, q) = 2 f + side
+  template <class Edge>
+  __device__ __forceinline__ void gather(const double *fhat, Edge &&edge, int ecount, int64_t F, int *err) {
     for (int i = threadIdx.x; i < EB * NF; i += blockDim.x) {
       const int el = i / NF, qk = i - el * NF;
       double v[M] = {0.0, 0.0, 0.0, 0.0};
       if (el < ecount) {
         const int q = qk / NE, k = qk - q * NE;
-        const int ef = elem_face[(size_t)(e0 + el) * 3 + q];
+        const int ef = edge(el, q);
         const int64_t f = checked(ef >> 1, F, err);
         const int side = ef & 1;
         const double *fp = fhat + ((size_t)f * NE + (side ? NE - 1 - k : k)) * M;
@@ -215,8 +223,9 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
 #pragma unroll
       for (int m = 0; m < M; ++m) sF[(el * RS + qk) * M + m] = v[m];
     }
-    __syncthreads();
+  }
 
+  __device__ __forceinline__ void lift() {
     // the lift's edge sums, in place of the element's fluxes of one variable:
     //   Q_a = sum_k omega_k P_a(xi_k) F0_k                            (face 0)
     //   G_even,k / G_odd,k = F1_k +/- F2_{NE-1-k}                   (faces 1, 2)
@@ -241,6 +250,10 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
       }
     }
 
+  }
+
+  // interpolation and the fluxes at the volume points; synchronised on return
+  __device__ __forceinline__ void points(const double *__restrict__ geo, int e0, int ecount, double gamma, int *err) {
     if constexpr (S::DIRECT) {
       // volume points: U = sum_j phi_j c_j, then G_r, G_s; one item per (element, point)
       for (int i = threadIdx.x; i < EB * NQ; i += blockDim.x) {
@@ -395,7 +408,12 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
         }
       }
       __syncthreads();
+    }
+  }
 
+  // the sums over the points of a row (collapsed grid); synchronised on return
+  __device__ __forceinline__ void row_sums() {
+    if constexpr (!S::DIRECT) {
       if constexpr (P >= 2 && P <= 4) {
         // Xa(a, ib) = sum_ia Ha wa P_a', Xb(a, ib) = sum_ia Hb wa P_a, one item per
         // (element, ib, variable) over every a, folded on the mirror pairs of the
@@ -497,7 +515,12 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
       __syncthreads();
 
     }
+  }
 
+  // update(el, j, acc, nv): the new values nv[M] of mode j of element el from the
+  // projection and lift acc[M]
+  template <class Update>
+  __device__ __forceinline__ void modes(int ecount, Update &&update) {
     // modes: V_j + lifted edge fluxes, 1/det J, stage update.  Sum-factorised:
     // the items of the modes with a >= 1 come first and those of the modes with
     // a = 0 (b = d) last, so that warps take one branch of the projection (for
@@ -560,40 +583,17 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
         }
       }
       double nv[M] = {0.0, 0.0, 0.0, 0.0};
-      if (el < ecount) {
-        const size_t e = (size_t)(e0 + el);
-        const double inv = geo[e * GEO + 4];
-        // stage update a0 u0 + b0 c + g dt R with R = acc / det J, as
-        // b0 c + a0 u0 + (g dt / det J) acc (and the second output alike)
-        const double kap = su.g * su.dt * inv;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          const size_t idx = (e * M + m) * NP + j;
-          double v;
-          if (mode == 0) {
-            v = acc[m] * inv;
-          } else {
-            double t = su.b0 * sC[(el * M + m) * NP + j];
-            if (su.a0 != 0.0) t = fma(su.a0, u0[idx], t);
-            v = fma(kap, acc[m], t);
-            if (su.out2) {
-              double t2 = su.y * v;
-              if (su.x != 0.0) t2 = fma(su.x, su.acc[idx], t2);
-              su.out2[idx] = fma(su.w * su.dt * inv, acc[m], t2);
-            }
-          }
-          out[idx] = v;
-          nv[m] = v;
-        }
-      }
+      if (el < ecount) update(el, j, acc, nv);
       // the new state, for the next stage's traces (sum-factorised: sH is free,
       // every thread has passed the barrier after the X phase, the last reader of
       // sH; direct: a buffer of its own, the modes still read sH)
 #pragma unroll
       for (int m = 0; m < M; ++m) sO[(el * M + m) * NP + j] = nv[m];
     }
+  }
 
-    if (trace_out) {
+  // the edge traces of the new state (synchronises before its first read)
+  __device__ __forceinline__ void traces(double *trace_out, int e0, int ecount) {
       __syncthreads();
       // Z_a of the new state (face 0 lies on beta = -1), one item per (element,
       // variable), in the buffer the modes have finished reading (sX; direct: sH)
@@ -619,8 +619,20 @@ __device__ __forceinline__ void element_sf_tiles(double *smem, const double *c, 
         dst[(NE + k) * M] = t1;
         dst[(3 * NE - 1 - k) * M] = t2;
       }
-    }
   }
+};
+
+// a0 u0 + b0 c + g dt R with R = acc / det J, as b0 c + a0 u0 + (g dt / det J) acc
+__device__ __forceinline__ double stage_value(const StageUpdate &su, double kap, double c, double u0, double acc) {
+  double t = su.b0 * c;
+  if (su.a0 != 0.0) t = fma(su.a0, u0, t);
+  return fma(kap, acc, t);
+}
+// x acc2 + y v + (w dt / det J) acc, the running sum of the classical RK4
+__device__ __forceinline__ double stage_sum(const StageUpdate &su, double inv, double v, double acc2, double acc) {
+  double t2 = su.y * v;
+  if (su.x != 0.0) t2 = fma(su.x, acc2, t2);
+  return fma(su.w * su.dt * inv, acc, t2);
 }
 
 template <int P, int NE, int Q>
@@ -630,10 +642,41 @@ k_element_sf(const double *c, const double *u0, double *out, double *__restrict_
              const int32_t *__restrict__ elem_face, DevTables tab, int N, int64_t F, StageUpdate su, int mode,
              double gamma, int *err) {
   extern __shared__ double smem[];
-  element_sf_tiles<P, NE, Q>(smem, c, u0, out, trace_out, fhat, geo, elem_face, tab, N, F, su, mode, gamma, err,
-                             blockIdx.x, gridDim.x);
+  SfTile<P, NE, Q> t(smem);
+  constexpr int NP = SfCfg<P, NE, Q>::NP, EB = SfCfg<P, NE, Q>::EB;
+  t.load_tables(tab);
+  const int ntiles = (N + EB - 1) / EB;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int e0 = tile * EB, ecount = min(EB, N - e0);
+    __syncthreads();
+    t.load_state(c, e0, ecount);
+    t.load_dirs(geo, e0, ecount);
+    t.gather(fhat, [&](int el, int q) { return elem_face[(size_t)(e0 + el) * 3 + q]; }, ecount, F, err);
+    __syncthreads();
+    t.lift();
+    t.points(geo, e0, ecount, gamma, err);
+    t.row_sums();
+    t.modes(ecount, [&](int el, int j, const double *acc, double *nv) {
+      const size_t e = (size_t)(e0 + el);
+      const double inv = geo[e * GEO + 4];
+      const double kap = su.g * su.dt * inv;
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const size_t idx = (e * M + m) * NP + j;
+        double v;
+        if (mode == 0) {
+          v = acc[m] * inv;
+        } else {
+          v = stage_value(su, kap, t.sC[(el * M + m) * NP + j], su.a0 != 0.0 ? u0[idx] : 0.0, acc[m]);
+          if (su.out2) su.out2[idx] = stage_sum(su, inv, v, su.x != 0.0 ? su.acc[idx] : 0.0, acc[m]);
+        }
+        out[idx] = v;
+        nv[m] = v;
+      }
+    });
+    if (trace_out) t.traces(trace_out, e0, ecount);
+  }
 }
-
 
 // CTAs of k_element_sf per SM (the kernel's shared memory attribute set first)
 template <int P, int NE, int Q>
@@ -688,38 +731,51 @@ int run_element_sf(const dg_mesh *m, const double *c, const double *u0, double *
 // launches (edge flux, element) do a few microseconds of work each and the step
 // is bound by launch latency (the paper's Section 7.1 finds its small meshes
 // alike).  This kernel runs every stage of a whole call inside one cooperative
-// launch: the edge phase (face_flux_points) and the element phase
-// (element_sf_tiles) of the same code as k_face and k_element_sf, separated by a
-// barrier over the grid, so the results are bitwise those of the separate
-// launches.
+// launch, one tile per block: the edge phase (face_flux_points) and the phases of
+// SfTile, the code of k_face and k_element_sf, with barriers over the grid between
+// them, so the results are bitwise those of the separate launches.
+//
+// A block keeps its tile's state, the step's first state, the classical RK4's
+// running sum, geometry and connectivity in shared memory from one stage to the
+// next; only traces and edge fluxes pass through memory.  The volume integral needs
+// neither, so it runs between a block's arrival at a barrier and its wait: the
+// points of the next stage behind the barrier after the traces, the row sums
+// behind the one after the edge fluxes.  (Cycles of a stage, p = 4, 800 elements:
+// 52,500 with whole barriers and the tile read back from memory at each stage, of
+// which 11,500 the barriers, 5,000 the loads and 11,000 the update that waited for
+// its operands.)
 // ---------------------------------------------------------------------------
 constexpr uint64_t kGridWaitNs = 2000000000ull;    // 2 s per barrier before giving up
 
-// All blocks of the (co-resident) grid meet here: one thread per block arrives on
-// a counter, the last one resets it and advances the generation the others
-// wait on.  The wait is bounded: after kGridWaitNs it records kErrTimeout and
-// returns false, and the caller leaves the kernel.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, int *err) {
-  __shared__ int ok_s;
+// A barrier over all blocks of the (co-resident) grid in two parts.  Arrival: the
+// block's writes so far, then one more on the counter; wait: until the counter
+// reaches target (nblocks times the barriers so far; it starts at 0).  The wait is
+// bounded: after kGridWaitNs it records kErrTimeout and returns false, and the
+// caller leaves the kernel.
+__device__ __forceinline__ void grid_arrive(unsigned *bar) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned *gen = bar + 1;
-    const unsigned g = *gen;
     __threadfence();                                  // this block's writes before its arrival
+    atomicAdd(bar, 1u);
+  }
+}
+__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned target, int *err) {
+  __shared__ int ok_s;
+  if (threadIdx.x == 0) {
     int ok = 1;
-    if (atomicAdd(bar, 1u) + 1u == nblocks) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const uint64_t t0 = tc::global_ns();
-      while (*gen == g) {
-        if (tc::global_ns() - t0 > kGridWaitNs) {
+    uint64_t t0 = 0;
+    for (unsigned it = 1;; ++it) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if ((it & 255u) == 0u) {
+        const uint64_t t = tc::global_ns();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > kGridWaitNs) {
           atomicOr(err, kErrTimeout);
           ok = 0;
           break;
         }
-        __nanosleep(32);
       }
     }
     __threadfence();                                  // the other blocks' writes after it
@@ -732,29 +788,91 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned nblocks, in
 constexpr int kSmallThreads = 128;
 constexpr int kSmallTiles[2] = {4, 8};          // elements per tile of the two variants
 
+// shared memory of the stepper: the tile's phases, then the step's first state and
+// the RK4 sum [EB][M][NP], 1/det J [EB] and the elements' edges [EB][3]
+template <int P, int NE, int Q, int EBX>
+struct SmallCfg {
+  using S = SfCfg<P, NE, Q, EBX>;
+  static constexpr int ROWS = S::EB * M * S::NP;
+  static constexpr int SMEM = S::SMEM + (2 * ROWS + S::EB) * 8 + (3 * S::EB + 1) / 2 * 8;
+};
+
 template <int P, int NE, int Q, int EBX>
 __global__ void __launch_bounds__(kSmallThreads, 4)
 k_rk_small(double *c, double *S, double *A, double *trace, double *fhat, const double *__restrict__ geo,
            const int32_t *__restrict__ elem_face, const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,
-           const FaceFix *__restrict__ ff, const double *__restrict__ bstate, const int32_t *__restrict__ elem_nbr, DevTables tab, int N, int64_t F,
-           GammaFix gf, double phi1, double dt, int nsteps, int method, int limit, unsigned *bar, int *err) {
+           const FaceFix *__restrict__ ff, const double *__restrict__ bstate, const int32_t *__restrict__ elem_nbr,
+           DevTables tab, int N, int64_t F, GammaFix gf, double phi1, double dt, int nsteps, int method, int limit, unsigned *bar, int *err) {
   extern __shared__ double smem[];
+  using Sm = SmallCfg<P, NE, Q, EBX>;
+  constexpr int NP = Sm::S::NP, EB = Sm::S::EB, ROWS = Sm::ROWS;
+  SfTile<P, NE, Q, EBX> t(smem);
+  double *sU0 = smem + Sm::S::SMEM / 8, *sA = sU0 + ROWS, *sInv = sA + ROWS;
+  int32_t *sEf = reinterpret_cast<int32_t *>(sInv + EB);
   const unsigned nb = gridDim.x;
+  unsigned target = 0;
   const int ns = rk_num_stages(method);
+  const int e0 = blockIdx.x * EB, ecount = min(EB, N - e0);
+
+  t.load_tables(tab);
+  t.load_state(c, e0, ecount);
+  for (int i = threadIdx.x; i < ecount * 3; i += blockDim.x) sEf[i] = elem_face[(size_t)e0 * 3 + i];
+  for (int i = threadIdx.x; i < ecount; i += blockDim.x) sInv[i] = geo[(size_t)(e0 + i) * GEO + 4];
+  __syncthreads();
+  t.load_dirs(geo, e0, ecount);
+  bool have_points = false;
   for (int step = 0; step < nsteps; ++step)
     for (int i = 0; i < ns; ++i) {
       const RkStage st = rk_stage(method, i, dt, c, S, A);
+      const bool last = step == nsteps - 1 && i == ns - 1;
+      if (i == 0)
+        for (int x = threadIdx.x; x < ROWS; x += blockDim.x) sU0[x] = t.sC[x];
       face_flux_points<NE>(trace, fhat, conn, fg, ff, bstate, N, F, gf, err, blockIdx.x, nb);
-      if (!grid_barrier(bar, nb, err)) return;
-      element_sf_tiles<P, NE, Q, EBX>(smem, st.cin, st.u0, st.out, trace, fhat, geo, elem_face, tab, N, F, st.su, 1,
-                                      gf.gamma, err, blockIdx.x, nb);
-      if (!grid_barrier(bar, nb, err)) return;
+      grid_arrive(bar);
+      target += nb;
+      if (!have_points) t.points(geo, e0, ecount, gf.gamma, err);
+      t.row_sums();
+      if (!grid_wait(bar, target, err)) return;
+      t.gather(fhat, [&](int el, int q) { return sEf[el * 3 + q]; }, ecount, F, err);
+      __syncthreads();
+      t.lift();
+      __syncthreads();
+      const double *u0 = method == DG_RK4 && i == 3 ? sA : sU0;
+      const StageUpdate &su = st.su;
+      t.modes(ecount, [&](int el, int j, const double *acc, double *nv) {
+        const double inv = sInv[el], kap = su.g * su.dt * inv;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          const int x = (el * M + m) * NP + j;
+          const double v = stage_value(su, kap, t.sC[x], u0[x], acc[m]);
+          if (su.out2) sA[x] = stage_sum(su, inv, v, sA[x], acc[m]);
+          if (limit || last) st.out[(size_t)e0 * M * NP + x] = v;
+          nv[m] = v;
+        }
+      });
+      t.traces(trace, e0, ecount);
+      if (last && !limit) return;
+      grid_arrive(bar);
+      target += nb;
+      have_points = !limit;
+      if (have_points) {
+        for (int x = threadIdx.x; x < ROWS; x += blockDim.x) t.sC[x] = x < ecount * M * NP ? t.sO[x] : 0.0;
+        __syncthreads();
+        t.points(geo, e0, ecount, gf.gamma, err);
+      }
+      if (!grid_wait(bar, target, err)) return;
       if constexpr (P == 1) {
         // with the limiter on, every stage value is limited in place (and the
-        // traces of the elements it limits rewritten) before the next stage
+        // traces of the elements it limits rewritten) before the next stage, which
+        // reads its tile back
         if (limit) {
           limit_p1_items<true>(st.out, trace, elem_nbr, tab.EPa, tab.EChiM1, tab.EChi, phi1, N, err, blockIdx.x, nb);
-          if (!grid_barrier(bar, nb, err)) return;
+          if (last) return;
+          grid_arrive(bar);
+          target += nb;
+          if (!grid_wait(bar, target, err)) return;
+          t.load_state(st.out, e0, ecount);
+          __syncthreads();
         }
       }
     }
@@ -771,7 +889,7 @@ const int *small_per_sm(int dev) {
   if (dev >= 0 && dev < 64 && ready.test(dev)) return r;
   auto k0 = k_rk_small<P, NE, Q, kSmallTiles[0]>;
   auto k1 = k_rk_small<P, NE, Q, kSmallTiles[1]>;
-  const int s0 = SfCfg<P, NE, Q, kSmallTiles[0]>::SMEM, s1 = SfCfg<P, NE, Q, kSmallTiles[1]>::SMEM;
+  const int s0 = SmallCfg<P, NE, Q, kSmallTiles[0]>::SMEM, s1 = SmallCfg<P, NE, Q, kSmallTiles[1]>::SMEM;
   r[0] = r[1] = 0;
   if (cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, s0) != cudaSuccess ||
       cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, s1) != cudaSuccess ||
@@ -798,7 +916,7 @@ int small_variant(const dg_mesh *m) {
 
 template <int P, int NE, int Q, int EBX>
 int run_rk_small(dg_mesh *m, double *c, double dt, int nsteps, int method, cudaStream_t s) {
-  using Sc = SfCfg<P, NE, Q, EBX>;
+  using Sc = SmallCfg<P, NE, Q, EBX>;
   auto kern = k_rk_small<P, NE, Q, EBX>;
   // one tile per block (the variant was chosen so that they are all resident);
   // the edge phase spreads its points over the same blocks

@@ -1,5 +1,5 @@
 """The split-product float64 element kernel (meshes too large for the fused
-small-mesh stepper, p >= 2) against the oracle, at the sizes where its tiling can
+small-mesh stepper) against the oracle, at the sizes where its tiling can
 go wrong: 7,442 elements leave 18 of 32 in the last tile, 8,192 none; every degree
 covers its batches of points and of contraction columns, both volume rules, each
 Runge-Kutta form of the update (one and two outputs), boundary faces, host-memory
@@ -18,7 +18,7 @@ from paper_1601_07944_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 
 EPS = 2.0 ** -53
-CASES = [(2, 0, "collapsed"), (3, 0, "collapsed"), (3, 3, "collapsed"), (4, 0, "collapsed"), (5, 0, "collapsed"),
+CASES = [(1, 0, "collapsed"), (1, 0, "symmetric"), (2, 0, "collapsed"), (3, 0, "collapsed"), (3, 3, "collapsed"), (4, 0, "collapsed"), (5, 0, "collapsed"),
          (2, 0, "symmetric"), (3, 0, "symmetric"), (3, 3, "symmetric"), (4, 0, "symmetric"), (5, 0, "symmetric")]
 
 
@@ -84,7 +84,7 @@ def test_boundary_faces(dgmod, oracle_mod, p):
     check_rhs(m, o, o.project_ic(I.steady_vortex))
 
 
-@pytest.mark.parametrize("p,rule", [(2, "collapsed"), (3, "collapsed"), (5, "collapsed"), (4, "symmetric")])
+@pytest.mark.parametrize("p,rule", [(1, "collapsed"), (2, "collapsed"), (3, "collapsed"), (5, "collapsed"), (4, "symmetric")])
 def test_host_state_and_repeats_same_bits(dgmod, p, rule):
     """The traces read from host memory, the ranges of the last stage and a second
     call after the state's own traces give the bits of plain one-step calls."""
@@ -102,6 +102,28 @@ def test_host_state_and_repeats_same_bits(dgmod, p, rule):
     torch.cuda.synchronize()
     assert torch.equal(a, b)
     assert torch.equal(a.cpu(), pinned)
+
+
+@pytest.mark.parametrize("rule", ["collapsed", "symmetric"])
+def test_limited_steps_same_bits(dgmod, oracle_mod, rule):
+    """p = 1 with every stage limited: the traces that the limiter rewrites are those
+    the next call forms, so two steps in one call and in two give the same bits."""
+    import torch
+    mesh = I.periodic_mesh(107)
+    m = dgmod.Mesh.from_mesh(mesh, 1, vol_rule=rule)
+    c = m.project_function(I.density_steps)
+    dt = I.fixed_dt(mesh, I.density_steps, 1)
+    m.set_limiter(True)
+    m.limit(c)
+    a, b = c.clone(), c.clone()
+    m.rk_step(a, dt, 2, method="rk2")
+    for _ in range(2):
+        m.rk_step(b, dt, 1, method="rk2")
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
+    o = oracle_mod.OracleDG.from_mesh(mesh, 1, vol_rule=rule)
+    o.set_limiter(True)
+    assert rel_l2(_host(a), o.rk2(c.cpu().numpy(), dt, 2)) < 1e-14
 
 
 def test_wide_range_rows(dgmod, oracle_mod):
