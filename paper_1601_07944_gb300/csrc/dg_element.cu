@@ -76,7 +76,16 @@ struct SfCfg {
   // third resident CTA per SM)
   static constexpr bool PREDIR = !DIRECT && P >= 3;
   static constexpr int DS = PREDIR ? 2 * (ND + 1) : 0;
-  static constexpr int TILE = EB * (M * NP + XS + 8 * NQ + RS * M + DS);
+  // SPREAD (the fused small-mesh stepper's tiles): a float64 instruction takes a
+  // warp as long with few lanes as with 32, and the tile leaves most lanes idle, so
+  // the lift, the modes and the mirror pairs go to more threads: one per variable
+  // and sum, one per mode and variable, one per point of a pair (where the items
+  // of the pairs and of the middle nodes fit in the block at once).
+  static constexpr bool SPREAD = EBX > 0;
+  static constexpr int NHALF = 2 * EB * ND * (ND / 2), MIDAT = (NHALF + 31) / 32 * 32;
+  static constexpr bool SPREAD_PAIRS = SPREAD && PAIRS && MIDAT + ((ND & 1) ? EB * ND : 0) <= 128;
+  static constexpr int LS = SPREAD ? LW : RS;               // stride of the lift sums
+  static constexpr int TILE = EB * (M * NP + XS + 8 * NQ + RS * M + DS + (SPREAD ? LW * M : 0));
   static constexpr int SMEM = (TAB + TILE) * 8;
   static_assert(DIRECT || 8 * NQ >= M * NP, "the new state reuses the point buffer");
 };
@@ -130,7 +139,7 @@ struct SfTile {
   using S = SfCfg<P, NE, Q, EBX>;
   static constexpr int NP = S::NP, ND = S::ND, NQ = S::NQ, NF = S::NF, EB = S::EB, RS = S::RS;
   double *sPa, *sPaW, *sdPaW, *sChi, *sChiA, *sdChiB, *sHalf, *sEChi, *sEWChi, *sEWPa, *sEChiM1, *sEPa;
-  double *sBvT, *sDr, *sDs, *sC, *sX, *sH, *sF, *sDir, *sO;
+  double *sBvT, *sDr, *sDs, *sC, *sX, *sH, *sF, *sDir, *sL, *sO;
 
   __device__ __forceinline__ explicit SfTile(double *smem) {
     sPa = smem;                  // [ND][ND]   P_a(alpha_ia)
@@ -153,6 +162,7 @@ struct SfTile {
     sH = sX + EB * S::XS;        // [EB][NQ][8]        Ha, Hb (direct: G_r, G_s); later the new state
     sF = sH + EB * NQ * 8;       // [EB][RS][M]        -F_hat_out * l, then the lift sums
     sDir = sF + EB * RS * M;     // [EB][ND+1][2]      J^tau row 0 + half_ia row 1 (ia < ND), row 1
+    sL = S::SPREAD ? sDir + EB * S::DS : sF;  // [EB][LS][M]  the lift sums (else in place of the fluxes)
     sO = S::DIRECT ? sX : sH;    // the new state
   }
 
@@ -231,25 +241,70 @@ struct SfTile {
     //   G_even,k / G_odd,k = F1_k +/- F2_{NE-1-k}                   (faces 1, 2)
     // so that the lift of mode j = (a, b) is
     //   chi_j(-1) Q_a + sum_k omega_k chi_j(xi_k) G_{a mod 2, k}
-    for (int i = threadIdx.x; i < EB * M; i += blockDim.x) {
-      double *fe = sF + (i / M) * RS * M + (i % M);
-      double f[NF];
+    if constexpr (S::SPREAD) {
+      for (int i = threadIdx.x; i < (ND + NE) * EB * M; i += blockDim.x) {
+        const int x = i / (EB * M), r = i - x * (EB * M);
+        const double *fe = sF + (r / M) * RS * M + (r % M);
+        double *lo = sL + (r / M) * S::LS * M + (r % M);
+        if (x < ND) {
+          double q = 0.0;
 #pragma unroll
-      for (int x = 0; x < NF; ++x) f[x] = fe[x * M];
-#pragma unroll
-      for (int a = 0; a < ND; ++a) {
-        double q = 0.0;
-#pragma unroll
-        for (int k = 0; k < NE; ++k) q = fma(sEWPa[a * NE + k], f[k], q);
-        fe[a * M] = q;
+          for (int k = 0; k < NE; ++k) q = fma(sEWPa[x * NE + k], fe[k * M], q);
+          lo[x * M] = q;
+        } else {
+          const int k = x - ND;
+          const double f1 = fe[(NE + k) * M], f2 = fe[(3 * NE - 1 - k) * M];
+          lo[x * M] = f1 + f2;
+          lo[(x + NE) * M] = f1 - f2;
+        }
       }
+    } else {
+      for (int i = threadIdx.x; i < EB * M; i += blockDim.x) {
+        double *fe = sF + (i / M) * RS * M + (i % M);
+        double f[NF];
 #pragma unroll
-      for (int k = 0; k < NE; ++k) {
-        fe[(ND + k) * M] = f[NE + k] + f[3 * NE - 1 - k];
-        fe[(ND + NE + k) * M] = f[NE + k] - f[3 * NE - 1 - k];
+        for (int x = 0; x < NF; ++x) f[x] = fe[x * M];
+#pragma unroll
+        for (int a = 0; a < ND; ++a) {
+          double q = 0.0;
+#pragma unroll
+          for (int k = 0; k < NE; ++k) q = fma(sEWPa[a * NE + k], f[k], q);
+          fe[a * M] = q;
+        }
+#pragma unroll
+        for (int k = 0; k < NE; ++k) {
+          fe[(ND + k) * M] = f[NE + k] + f[3 * NE - 1 - k];
+          fe[(ND + NE + k) * M] = f[NE + k] - f[3 * NE - 1 - k];
+        }
       }
     }
+  }
 
+  // the x-th (element, ib) at the middle node alpha = 0 of an odd number of nodes,
+  // where P_a(0) = 0 for odd a
+  __device__ __forceinline__ void middle_node(int x, int ecount, double gamma, int *err) {
+    const int el = x / ND, ib = x - el * ND;
+    constexpr int MID = ND / 2;
+    const double *w0 = sX + ((el * ND) * ND + ib) * 8;
+    double U[M] = {w0[0], w0[1], w0[2], w0[3]};
+#pragma unroll
+    for (int a = 2; a < ND; a += 2) {
+      const double pa = sPa[a * ND + MID];
+      const double *w = sX + ((el * ND + a) * ND + ib) * 8;
+#pragma unroll
+      for (int m = 0; m < M; ++m) U[m] = fma(pa, w[m], U[m]);
+    }
+    double Ha[M], Hb[M];
+    if (el < ecount) {
+      const double *dir = sDir + el * 2 * (ND + 1);
+      flux_two_dirs(U, dir[2 * MID], dir[2 * MID + 1], dir[2 * ND], dir[2 * ND + 1], gamma, err, Ha, Hb);
+    } else {
+#pragma unroll
+      for (int m = 0; m < M; ++m) { Ha[m] = 0.0; Hb[m] = 0.0; }
+    }
+    double *h = sH + ((size_t)el * NQ + ib * ND + MID) * 8;
+#pragma unroll
+    for (int m = 0; m < M; ++m) { h[m] = Ha[m]; h[4 + m] = Hb[m]; }
   }
 
   // interpolation and the fluxes at the volume points; synchronised on return
@@ -302,34 +357,56 @@ struct SfTile {
       // point slots of the pair receive the sums and differences the folded
       // projection takes: slot ia (Ha + Ha', Hb + Hb'), slot ia' (Ha - Ha',
       // Hb - Hb'); the middle slot keeps (Ha, Hb).
-      if constexpr (S::PAIRS) {
+      if constexpr (S::SPREAD_PAIRS) {
+        // a thread per point of a pair (neighbouring lanes), the middle nodes in
+        // warps of their own: the sums of the form below, each formed by both
+        // threads of a pair or by one of them
+        constexpr int NH = ND / 2;
+        const int i = threadIdx.x;
+        if (i < S::NHALF) {
+          const int left = S::NHALF - (i & ~31);
+          const unsigned mask = left >= 32 ? 0xFFFFFFFFu : (1u << left) - 1u;
+          const int hf = i & 1, pr = i >> 1;
+          const int el = pr / (ND * NH), r = pr - el * (ND * NH), ib = r / NH, ia = r - ib * NH;
+          const int ia2 = ND - 1 - ia;
+          const double *w0 = sX + ((el * ND) * ND + ib) * 8;
+          double E[M] = {w0[0], w0[1], w0[2], w0[3]}, O[M];
+#pragma unroll
+          for (int a = 1; a < ND; ++a) {
+            const double pa = sPa[a * ND + ia];
+            const double *w = sX + ((el * ND + a) * ND + ib) * 8;
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+              if (a == 1) O[m] = pa * w[m];
+              else if (a & 1) O[m] = fma(pa, w[m], O[m]);
+              else E[m] = fma(pa, w[m], E[m]);
+            }
+          }
+          double Ha[M] = {0.0, 0.0, 0.0, 0.0}, Hb[M] = {0.0, 0.0, 0.0, 0.0};
+          if (el < ecount) {
+            double U[M];
+#pragma unroll
+            for (int m = 0; m < M; ++m) U[m] = hf ? E[m] - O[m] : E[m] + O[m];
+            const double *dir = sDir + el * 2 * (ND + 1), *da = dir + 2 * (hf ? ia2 : ia);
+            flux_two_dirs(U, da[0], da[1], dir[2 * ND], dir[2 * ND + 1], gamma, err, Ha, Hb);
+          }
+          double *h = sH + ((size_t)el * NQ + ib * ND + (hf ? ia2 : ia)) * 8;
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            const double oa = __shfl_xor_sync(mask, Ha[m], 1), ob = __shfl_xor_sync(mask, Hb[m], 1);
+            h[m] = hf ? __dsub_rn(oa, Ha[m]) : __dadd_rn(Ha[m], oa);
+            h[4 + m] = hf ? __dsub_rn(ob, Hb[m]) : __dadd_rn(Hb[m], ob);
+          }
+        } else if ((ND & 1) && i >= S::MIDAT && i < S::MIDAT + EB * ND) {
+          middle_node(i - S::MIDAT, ecount, gamma, err);
+        }
+      } else if constexpr (S::PAIRS) {
         constexpr int NH = ND / 2, NPAIR = EB * ND * NH, NMID = (ND & 1) ? EB * ND : 0;
         for (int i = threadIdx.x; i < NPAIR + NMID; i += blockDim.x) {
           if ((ND & 1) && i >= NPAIR) {
             // the middle node alpha = 0 (p + 1 odd), after all the pairs so that
-            // warps stay uniform: P_a(0) = 0 for odd a
-            const int el = (i - NPAIR) / ND, ib = (i - NPAIR) - el * ND;
-            constexpr int MID = ND / 2;
-            const double *w0 = sX + ((el * ND) * ND + ib) * 8;
-            double U[M] = {w0[0], w0[1], w0[2], w0[3]};
-#pragma unroll
-            for (int a = 2; a < ND; a += 2) {
-              const double pa = sPa[a * ND + MID];
-              const double *w = sX + ((el * ND + a) * ND + ib) * 8;
-#pragma unroll
-              for (int m = 0; m < M; ++m) U[m] = fma(pa, w[m], U[m]);
-            }
-            double Ha[M], Hb[M];
-            if (el < ecount) {
-              const double *dir = sDir + el * 2 * (ND + 1);
-              flux_two_dirs(U, dir[2 * MID], dir[2 * MID + 1], dir[2 * ND], dir[2 * ND + 1], gamma, err, Ha, Hb);
-            } else {
-#pragma unroll
-              for (int m = 0; m < M; ++m) { Ha[m] = 0.0; Hb[m] = 0.0; }
-            }
-            double *h = sH + ((size_t)el * NQ + ib * ND + MID) * 8;
-#pragma unroll
-            for (int m = 0; m < M; ++m) { h[m] = Ha[m]; h[4 + m] = Hb[m]; }
+            // warps stay uniform
+            middle_node(i - NPAIR, ecount, gamma, err);
             continue;
           }
           const int el = i / (ND * NH), r = i - el * (ND * NH), ib = r / NH, ia = r - ib * NH;
@@ -360,8 +437,10 @@ struct SfTile {
             flux_two_dirs(U, dir[2 * ia2], dir[2 * ia2 + 1], bx, by, gamma, err, Ha2, Hb2);
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-              S1[m] = Ha[m] + Ha2[m]; D1[m] = Ha[m] - Ha2[m];
-              S2[m] = Hb[m] + Hb2[m]; D2[m] = Hb[m] - Hb2[m];
+              // (not contracted with the products they add: SPREAD_PAIRS adds them
+              // in another thread than the one that formed them)
+              S1[m] = __dadd_rn(Ha[m], Ha2[m]); D1[m] = __dsub_rn(Ha[m], Ha2[m]);
+              S2[m] = __dadd_rn(Hb[m], Hb2[m]); D2[m] = __dsub_rn(Hb[m], Hb2[m]);
             }
           } else {
 #pragma unroll
@@ -517,90 +596,94 @@ struct SfTile {
     }
   }
 
-  // update(el, j, acc, nv): the new values nv[M] of mode j of element el from the
-  // projection and lift acc[M]
+  // update(el, j, m, acc): the new value of mode j, variable m of element el from its
+  // projection and lift acc
   template <class Update>
   __device__ __forceinline__ void modes(int ecount, Update &&update) {
-    // modes: V_j + lifted edge fluxes, 1/det J, stage update.  Sum-factorised:
-    // the items of the modes with a >= 1 come first and those of the modes with
-    // a = 0 (b = d) last, so that warps take one branch of the projection (for
-    // a = 0, Xa(0, .) = 0 and only the Xb term is formed)
-    for (int i = threadIdx.x; i < EB * NP; i += blockDim.x) {
+    // V_j + lifted edge fluxes, then the caller's update.  Sum-factorised: the items
+    // of the modes with a >= 1 come first and those of the modes with a = 0 (b = d)
+    // last, so that warps take one branch of the projection (for a = 0,
+    // Xa(0, .) = 0 and only the Xb term is formed).  An item has all four variables;
+    // SPREAD: one.
+    constexpr int NV = S::SPREAD ? 1 : M, IV = M / NV;
+    for (int i = threadIdx.x; i < EB * NP * IV; i += blockDim.x) {
+      const int it = i / IV, m0 = i - it * IV;
       int el, j;
       if constexpr (S::DIRECT) {
-        el = i / NP;
-        j = i - el * NP;
+        el = it / NP;
+        j = it - el * NP;
       } else {
         constexpr int NB = NP - ND;                   // modes with a >= 1
-        if (i < EB * NB) {
-          el = i / NB;
-          j = mode_a_ge1(i - el * NB);
+        if (it < EB * NB) {
+          el = it / NB;
+          j = mode_a_ge1(it - el * NB);
         } else {
-          const int i2 = i - EB * NB;
+          const int i2 = it - EB * NB;
           el = i2 / ND;
           const int d = i2 - el * ND;
           j = d * (d + 1) / 2 + d;
         }
       }
       const int a = mode_a(j);
-      double acc[M] = {0.0, 0.0, 0.0, 0.0};
+      double acc[NV];
+#pragma unroll
+      for (int m = 0; m < NV; ++m) acc[m] = 0.0;
       if constexpr (S::DIRECT) {
 #pragma unroll
         for (int k = 0; k < NQ; ++k) {
           const double dr = sDr[k * NP + j], ds = sDs[k * NP + j];
-          const double *h = sH + (el * NQ + k) * 8;
+          const double *h = sH + (el * NQ + k) * 8 + m0;
 #pragma unroll
-          for (int m = 0; m < M; ++m) acc[m] = fma(ds, h[4 + m], fma(dr, h[m], acc[m]));
+          for (int m = 0; m < NV; ++m) acc[m] = fma(ds, h[4 + m], fma(dr, h[m], acc[m]));
         }
       } else if (a > 0) {
 #pragma unroll
         for (int ib = 0; ib < ND; ++ib) {
           const double ch = sChiA[j * ND + ib], dch = sdChiB[j * ND + ib];
-          const double *x = sX + ((el * ND + a) * ND + ib) * 8;
+          const double *x = sX + ((el * ND + a) * ND + ib) * 8 + m0;
 #pragma unroll
-          for (int m = 0; m < M; ++m) acc[m] = fma(dch, x[4 + m], fma(ch, x[m], acc[m]));
+          for (int m = 0; m < NV; ++m) acc[m] = fma(dch, x[4 + m], fma(ch, x[m], acc[m]));
         }
       } else {
 #pragma unroll
         for (int ib = 0; ib < ND; ++ib) {
           const double dch = sdChiB[j * ND + ib];
-          const double *x = sX + (el * ND * ND + ib) * 8;
+          const double *x = sX + (el * ND * ND + ib) * 8 + m0;
 #pragma unroll
-          for (int m = 0; m < M; ++m) acc[m] = fma(dch, x[4 + m], acc[m]);
+          for (int m = 0; m < NV; ++m) acc[m] = fma(dch, x[4 + m], acc[m]);
         }
       }
       {
-        const double *fl = sF + el * RS * M;
+        const double *fl = sL + el * S::LS * M + m0;
         const double c1 = sEChiM1[j];
 #pragma unroll
-        for (int m = 0; m < M; ++m) acc[m] = fma(c1, fl[a * M + m], acc[m]);
+        for (int m = 0; m < NV; ++m) acc[m] = fma(c1, fl[a * M + m], acc[m]);
         const double *g = fl + (ND + (a & 1) * NE) * M;
 #pragma unroll
         for (int k = 0; k < NE; ++k) {
           const double l = sEWChi[j * NE + k];
 #pragma unroll
-          for (int m = 0; m < M; ++m) acc[m] = fma(l, g[k * M + m], acc[m]);
+          for (int m = 0; m < NV; ++m) acc[m] = fma(l, g[k * M + m], acc[m]);
         }
       }
-      double nv[M] = {0.0, 0.0, 0.0, 0.0};
-      if (el < ecount) update(el, j, acc, nv);
       // the new state, for the next stage's traces (sum-factorised: sH is free,
-      // every thread has passed the barrier after the X phase, the last reader of
+      // every thread has passed the barrier after the row sums, the last reader of
       // sH; direct: a buffer of its own, the modes still read sH)
 #pragma unroll
-      for (int m = 0; m < M; ++m) sO[(el * M + m) * NP + j] = nv[m];
+      for (int m = 0; m < NV; ++m)
+        sO[(el * M + m0 + m) * NP + j] = el < ecount ? update(el, j, m0 + m, acc[m]) : 0.0;
     }
   }
 
-  // the edge traces of the new state (synchronises before its first read)
-  __device__ __forceinline__ void traces(double *trace_out, int e0, int ecount) {
+  // the edge traces of the state sS, sO or sC (synchronises before its first read)
+  __device__ __forceinline__ void traces(const double *sS, double *trace_out, int e0, int ecount) {
       __syncthreads();
       // Z_a of the new state (face 0 lies on beta = -1), one item per (element,
       // variable), in the buffer the modes have finished reading (sX; direct: sH)
       double *sZ = S::DIRECT ? sH : sX;
       for (int i = threadIdx.x; i < ecount * M; i += blockDim.x) {
         double z[ND + 1];
-        face_sums<P>(sO + i * NP, sEChiM1, sEChi[0], z);
+        face_sums<P>(sS + i * NP, sEChiM1, sEChi[0], z);
 #pragma unroll
         for (int a = 0; a <= ND; ++a) sZ[i * (ND + 1) + a] = z[a];
       }
@@ -611,7 +694,7 @@ struct SfTile {
       //   Y_a(xi) = sum_b chi_ab(xi) c_ab
       for (int i = threadIdx.x; i < ecount * M * NE; i += blockDim.x) {
         const int el = i / (M * NE), m = (i / NE) % M, k = i % NE;
-        const double *cj = sO + (el * M + m) * NP;
+        const double *cj = sS + (el * M + m) * NP;
         double *dst = trace_out + (size_t)(e0 + el) * NF * M + m;
         double t0, t1, t2;
         edge_traces_unit<P, NE>(cj, sZ + (el * M + m) * (ND + 1), sEPa, sEChi, k, t0, t1, t2);
@@ -656,25 +739,21 @@ k_element_sf(const double *c, const double *u0, double *out, double *__restrict_
     t.lift();
     t.points(geo, e0, ecount, gamma, err);
     t.row_sums();
-    t.modes(ecount, [&](int el, int j, const double *acc, double *nv) {
-      const size_t e = (size_t)(e0 + el);
+    t.modes(ecount, [&](int el, int j, int m, double acc) {
+      const size_t e = (size_t)(e0 + el), idx = (e * M + m) * NP + j;
       const double inv = geo[e * GEO + 4];
       const double kap = su.g * su.dt * inv;
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const size_t idx = (e * M + m) * NP + j;
-        double v;
-        if (mode == 0) {
-          v = acc[m] * inv;
-        } else {
-          v = stage_value(su, kap, t.sC[(el * M + m) * NP + j], su.a0 != 0.0 ? u0[idx] : 0.0, acc[m]);
-          if (su.out2) su.out2[idx] = stage_sum(su, inv, v, su.x != 0.0 ? su.acc[idx] : 0.0, acc[m]);
-        }
-        out[idx] = v;
-        nv[m] = v;
+      double v;
+      if (mode == 0) {
+        v = acc * inv;
+      } else {
+        v = stage_value(su, kap, t.sC[(el * M + m) * NP + j], su.a0 != 0.0 ? u0[idx] : 0.0, acc);
+        if (su.out2) su.out2[idx] = stage_sum(su, inv, v, su.x != 0.0 ? su.acc[idx] : 0.0, acc);
       }
+      out[idx] = v;
+      return v;
     });
-    if (trace_out) t.traces(trace_out, e0, ecount);
+    if (trace_out) t.traces(t.sO, trace_out, e0, ecount);
   }
 }
 
@@ -778,7 +857,6 @@ __device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned target, int *e
         }
       }
     }
-    __threadfence();                                  // the other blocks' writes after it
     ok_s = ok;
   }
   __syncthreads();
@@ -820,7 +898,12 @@ k_rk_small(double *c, double *S, double *A, double *trace, double *fhat, const d
   for (int i = threadIdx.x; i < ecount; i += blockDim.x) sInv[i] = geo[(size_t)(e0 + i) * GEO + 4];
   __syncthreads();
   t.load_dirs(geo, e0, ecount);
-  bool have_points = false;
+  t.traces(t.sC, trace, e0, ecount);
+  grid_arrive(bar);
+  target += nb;
+  t.points(geo, e0, ecount, gf.gamma, err);
+  if (!grid_wait(bar, target, err)) return;
+  bool have_points = true;
   for (int step = 0; step < nsteps; ++step)
     for (int i = 0; i < ns; ++i) {
       const RkStage st = rk_stage(method, i, dt, c, S, A);
@@ -839,18 +922,15 @@ k_rk_small(double *c, double *S, double *A, double *trace, double *fhat, const d
       __syncthreads();
       const double *u0 = method == DG_RK4 && i == 3 ? sA : sU0;
       const StageUpdate &su = st.su;
-      t.modes(ecount, [&](int el, int j, const double *acc, double *nv) {
+      t.modes(ecount, [&](int el, int j, int m, double acc) {
         const double inv = sInv[el], kap = su.g * su.dt * inv;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          const int x = (el * M + m) * NP + j;
-          const double v = stage_value(su, kap, t.sC[x], u0[x], acc[m]);
-          if (su.out2) sA[x] = stage_sum(su, inv, v, sA[x], acc[m]);
-          if (limit || last) st.out[(size_t)e0 * M * NP + x] = v;
-          nv[m] = v;
-        }
+        const int x = (el * M + m) * NP + j;
+        const double v = stage_value(su, kap, t.sC[x], u0[x], acc);
+        if (su.out2) sA[x] = stage_sum(su, inv, v, sA[x], acc);
+        if (limit || last) st.out[(size_t)e0 * M * NP + x] = v;
+        return v;
       });
-      t.traces(trace, e0, ecount);
+      t.traces(t.sO, trace, e0, ecount);
       if (last && !limit) return;
       grid_arrive(bar);
       target += nb;

@@ -268,8 +268,7 @@ int launch_split_sym(const dg_mesh *m, const double *c, const double *u0, double
 int split_wave(const dg_mesh *m);      // tiles (of 32 elements) in flight on the GPU
 int launch_convert_check(int n, unsigned long long *bad, void *stream);
 // The fused small-mesh stepper (float64; the limiter a phase of it when on):
-// nsteps steps of `method` on c in one cooperative launch, the traces of c
-// already in m->trace.  Returns a
+// nsteps steps of `method` on c in one cooperative launch.  Returns a
 // cudaError_t cast to int.  small_rk_fits: whether the mesh is small enough (its
 // element tiles fit in one wave of the GPU).
 bool small_rk_fits(const dg_mesh *m);
