@@ -26,7 +26,7 @@ constexpr int GEO = 8;
 
 // Face record: left element, its local face, right element, its local face; on a
 // boundary face r is the boundary code (DG_BC_WALL, DG_BC_STATE) and R = -1.
-struct FaceConn { int32_t l, L, r, R; };
+struct alignas(16) FaceConn { int32_t l, L, r, R; };
 // Face geometry (8 doubles): unit normal n (left -> right) and half length l
 // (Eq. len); then the products the edge flux uses, formed once on the host with
 // h = l / 2: hk = h^2 gamma (gamma - 1), the scaled normal s = h n, and (gamma - 1) s.

@@ -58,7 +58,8 @@ k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *
     const FaceConn cn = conn[f];
     const FaceGeo *g = fg + f;
     const FaceFix fix = ff[f];
-    const double sx = g->sx, sy = g->sy;
+    const double2 s2 = *reinterpret_cast<const double2 *>(&g->sx);
+    const double sx = s2.x, sy = s2.y;
     // [N][NF][M] float32: one point's four values are one aligned float4
     constexpr bool bnd = BND;
     const int64_t el = checked(cn.l, N, err);
