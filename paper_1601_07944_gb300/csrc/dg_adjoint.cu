@@ -633,6 +633,26 @@ k_adj_combine_sf(const double *__restrict__ uvol, const double *__restrict__ TB,
   }
 }
 
+template <int NE>
+int run_adj_face(const dg_mesh *m, const double *T, const double *G, double *TB, cudaStream_t st) {
+  const int64_t nf = m->F * NE;
+  k_adj_face<NE><<<(int)((nf + kThreads - 1) / kThreads), kThreads, 0, st>>>(T, G, TB, m->face_conn, m->face_geo,
+                                                                             m->bstate, m->N, m->F, m->gamma,
+                                                                             m->err_flag);
+  return (int)cudaGetLastError();
+}
+
+// on the meshes of the split-product kernels (dg_adj_split.cu)
+template <int NE>
+int run_adj_split(const dg_mesh *m, const double *u, const double *lam, double *uvol, double *G, double *T, double *TB,
+                  const double *X, const double *Y, const double *Z, double x0, double x1, double x2, double s,
+                  double *out, cudaStream_t st) {
+  int e = launch_adj_split(m, u, lam, uvol, G, T, st);
+  if (e == (int)cudaSuccess) e = run_adj_face<NE>(m, T, G, TB, st);
+  if (e == (int)cudaSuccess) e = launch_adj_sum_split(m, uvol, TB, X, Y, Z, x0, x1, x2, s, out, st);
+  return e;
+}
+
 template <int P, int NE>
 int run_adj_sf(const dg_mesh *m, const double *u, const double *lam, double *uvol, double *G, double *T, double *TB,
                const double *X, const double *Y, const double *Z, double x0, double x1, double x2, double s,
@@ -654,11 +674,7 @@ int run_adj_sf(const dg_mesh *m, const double *u, const double *lam, double *uvo
   int grid = ntiles < m->num_sms * per_sm ? ntiles : m->num_sms * per_sm;
   k_adj_element_sf<P, NE><<<grid, kThreads, A::SMEM, st>>>(u, lam, uvol, G, T, m->geo, m->tab, (int)m->N, m->gamma);
   if ((e = cudaGetLastError()) != cudaSuccess) return (int)e;
-  const int64_t nf = m->F * NE;
-  k_adj_face<NE><<<(int)((nf + kThreads - 1) / kThreads), kThreads, 0, st>>>(T, G, TB, m->face_conn, m->face_geo,
-                                                                             m->bstate, m->N, m->F, m->gamma,
-                                                                             m->err_flag);
-  if ((e = cudaGetLastError()) != cudaSuccess) return (int)e;
+  if ((e = (cudaError_t)run_adj_face<NE>(m, T, G, TB, st)) != cudaSuccess) return (int)e;
   grid = ntiles < m->num_sms * 4 ? ntiles : m->num_sms * 4;
   k_adj_combine_sf<P, NE><<<grid, kThreads, 0, st>>>(uvol, TB, m->tab, X, Y, Z, x0, x1, x2, s, out, (int)m->N);
   return (int)cudaGetLastError();
@@ -688,11 +704,7 @@ int run_adj(const dg_mesh *m, const double *u, const double *lam, double *uvol, 
   int grid = ntiles < m->num_sms * per_sm ? ntiles : m->num_sms * per_sm;
   k_adj_element<P, NE, Q><<<grid, kThreads, A::SMEM, st>>>(u, lam, uvol, G, T, m->geo, m->tab, (int)m->N, m->gamma);
   if ((e = cudaGetLastError()) != cudaSuccess) return (int)e;
-  const int64_t nf = m->F * NE;
-  k_adj_face<NE><<<(int)((nf + kThreads - 1) / kThreads), kThreads, 0, st>>>(T, G, TB, m->face_conn, m->face_geo,
-                                                                             m->bstate, m->N, m->F, m->gamma,
-                                                                             m->err_flag);
-  if ((e = cudaGetLastError()) != cudaSuccess) return (int)e;
+  if ((e = (cudaError_t)run_adj_face<NE>(m, T, G, TB, st)) != cudaSuccess) return (int)e;
   grid = ntiles < m->num_sms * 4 ? ntiles : m->num_sms * 4;
   k_adj_combine<P, NE><<<grid, kThreads, 0, st>>>(uvol, TB, m->tab.BfT, X, Y, Z, x0, x1, x2, s, out, (int)m->N);
   return (int)cudaGetLastError();
@@ -705,7 +717,9 @@ int launch_rhs_vjp(const dg_mesh *m, const double *u, const double *lam, double 
                    double x2, double s, double *out, void *stream) {
   cudaStream_t st = (cudaStream_t)stream;
 #define CALL(P, NE)                                                                                  \
-  (m->rule == DG_RULE_SYMMETRIC                                                                      \
+  (m->adj_split_img                                                                                  \
+       ? run_adj_split<NE>(m, u, lam, uvol, G, T, TB, X, Y, Z, x0, x1, x2, s, out, st)               \
+   : m->rule == DG_RULE_SYMMETRIC                                                                    \
        ? run_adj<P, NE, sym_points(P)>(m, u, lam, uvol, G, T, TB, X, Y, Z, x0, x1, x2, s, out, st)  \
        : run_adj_sf<P, NE>(m, u, lam, uvol, G, T, TB, X, Y, Z, x0, x1, x2, s, out, st))
   if (m->p == 1 && m->ne == 2) return CALL(1, 2);

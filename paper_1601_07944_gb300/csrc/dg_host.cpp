@@ -414,6 +414,7 @@ void free_mesh(dg_mesh *m) {
   cudaFree(m->gbar);
   cudaFree(m->tc_img[0]); cudaFree(m->tc_img[1]);
   cudaFree(m->split_img);
+  cudaFree(m->adj_split_img);
   if (m->copy_stream) cudaStreamDestroy(m->copy_stream);
   for (auto &e : m->copy_ev)
     if (e) cudaEventDestroy(e);
@@ -1316,6 +1317,12 @@ static dg_status adjoint_buffers(dg_mesh *m, const char *who) {
     cudaError_t e = cudaMalloc(&m->adj_buf, sizeof(double) * need);
     if (e != cudaSuccess) { cudaGetLastError(); return fail(DG_ENOMEM, "%s: cudaMalloc", who); }
     m->adj_doubles = need;
+    if (!m->adj_split_img && (e = (cudaError_t)dg::adj_split_tables(m)) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(m->adj_split_img);
+      m->adj_split_img = nullptr;
+      return fail(DG_ECUDA, "%s: tables: %s", who, cudaGetErrorString(e));
+    }
   }
   return DG_OK;
 }

@@ -201,6 +201,7 @@ struct dg_mesh {
   unsigned *gbar;              // [2] grid barrier of the fused small-mesh stepper (count, generation)
   unsigned char *tc_img[2];    // B operand images of the tensor-core kernel (1xTF32, 3xTF32)
   unsigned char *split_img;    // table digits of the split-product float64 kernel; null: the mesh does not use it
+  unsigned char *adj_split_img;   // the same for the adjoint's kernels; null: not used
   int small_stepper;           // dg_set_small_mesh_stepper (on by default)
   cudaStream_t copy_stream;    // dg_rk_step_host's copies out (created on first use)
   cudaEvent_t copy_ev[2];
@@ -266,6 +267,14 @@ int launch_split_sym(const dg_mesh *m, const double *c, const double *u0, double
                      const double *fhat, const StageUpdate &su, int mode, double *copy, void *stream, int64_t e0,
                      int64_t e1);
 int split_wave(const dg_mesh *m);      // tiles (of 32 elements) in flight on the GPU
+// The adjoint's element kernels on the same meshes, p <= 3 (dg_adj_split.cu):
+// adj_split_tables builds m->adj_split_img on the first adjoint call (synchronous);
+// launch_adj_split and launch_adj_sum_split are launch_rhs_vjp's first and last part.
+int adj_split_tables(dg_mesh *m);
+int launch_adj_split(const dg_mesh *m, const double *u, const double *lam, double *uvol, double *G, double *T,
+                     void *stream);
+int launch_adj_sum_split(const dg_mesh *m, const double *uvol, const double *TB, const double *X, const double *Y,
+                         const double *Z, double x0, double x1, double x2, double s, double *out, void *stream);
 int launch_convert_check(int n, unsigned long long *bad, void *stream);
 // The fused small-mesh stepper (float64; the limiter a phase of it when on):
 // nsteps steps of `method` on c in one cooperative launch.  Returns a

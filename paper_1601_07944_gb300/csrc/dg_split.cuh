@@ -42,7 +42,7 @@
  * each cuts half of the row's K slots and reassembles half of its outputs.  A CTA
  * holds three groups (two at p = 5: shared memory) with barriers of their own that
  * share one copy of the tables, so that one group's integer phases run beside
- * another's flux phase (split_groups, flux_turn).  Per tile:
+ * another's flux phase (split_groups, take_turn).  Per tile:
  *   GEMM 1  U  = c Phi           interpolation to the volume points
  *           float64 Euler flux, one (element, point) item per thread
  *   GEMM 2  D  = [G_r | G_s | lifted fluxes] [Dr; Ds; Lf]   projection and lift
@@ -231,6 +231,20 @@ __device__ __forceinline__ void gemm_digits(uint32_t d, uint32_t a, int ca, uint
 
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
+// One group of the CTA in the float64 phase at a time: the float64 pipe serves one
+// group as fast as two, and taking turns keeps the groups out of step, so that
+// one's integer phases run beside another's flux (two groups, p = 3: 0.221 against
+// 0.274 ms without turns; three groups: 0.202, two of them at once 0.214).  A wait
+// that does not end soon goes ahead (the order is for speed only); the holder sets
+// *turn to 0 after the phase.
+__device__ __forceinline__ void take_turn(int *turn, int tid) {
+  if (tid != 0) return;
+  for (int i = 0; i < 400; ++i) {
+    if (atomicCAS(turn, 0, 1) == 0) break;
+    __nanosleep(64);
+  }
+}
+
 // -x/2 of a normal x on the bit pattern (a float64 multiply would take a slot of
 // the float64 pipe)
 __device__ __forceinline__ double neg_half_bits(double x) {
@@ -368,18 +382,6 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
     bar_sync(1 + T::SUBS + sub * 4 + quarter, 64);
     return max(v, s[(h ^ 1) * 128 + row]);
   };
-  // One group of the CTA in the flux phase at a time: the float64 pipe serves one
-  // group as fast as two, and taking turns keeps the groups out of step, so that
-  // one's integer phases run beside another's flux (two groups, p = 3: 0.221 against
-  // 0.274 ms without turns; three groups: 0.202, two of them at once 0.214).  A wait
-  // that does not end soon goes ahead (the order is for speed only).
-  auto flux_turn = [&]() {
-    if (tid != 0) return;
-    for (int i = 0; i < 400; ++i) {
-      if (atomicCAS(turn, 0, 1) == 0) break;
-      __nanosleep(64);
-    }
-  };
   // this half's NPH values -> A columns of GEMMs 1 and 3
   auto store_modes = [&](const double *v, int E) {
 #pragma unroll
@@ -494,7 +496,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
           }
         }
         tc::fence_before_sync();
-        if (b == T::NB1 - 1) flux_turn();
+        if (b == T::NB1 - 1) take_turn(turn, tid);
         if (!sub_sync()) return false;
         tc::fence_after_sync();
       }

@@ -201,3 +201,44 @@ def test_edge_flux_range(dgmod, oracle_mod, p, ic):
         wave = np.linalg.norm(c[:, k] / np.sqrt(det[:, 0])) * 10.0 * max(1.0, np.sqrt(np.max(np.abs(c[:, 3] / c[:, :1, 0][:, 0:1]))))
         assert np.linalg.norm(got[:, k] - ref[:, k]) <= 1e-12 * scale + 16 * EPS * (scale + wave)
     m.device_status()
+
+
+# The adjoint's kernels of the same meshes (p <= 3) against the oracle's reverse
+# sweep: 1e-12 relative, as for the float64 kernels they replace, on states with the
+# small noise of the other adjoint tests: on the unperturbed stream (1, 1) the normal
+# velocity vanishes on the mesh's diagonals, and the derivative of its magnitude there
+# is the sign of a rounding error.
+@pytest.mark.parametrize("n", [61, 64])
+@pytest.mark.parametrize("p,ne,rule", [c for c in CASES if c[0] <= 3])
+def test_adjoint(dgmod, oracle_mod, p, ne, rule, n):
+    mesh = I.periodic_mesh(n)
+    m = dgmod.Mesh.from_mesh(mesh, p, n_edge_pts=ne, vol_rule=rule)
+    o = oracle_mod.OracleDG.from_mesh(mesh, p, n_edge_pts=ne, vol_rule=rule)
+    rng = np.random.default_rng(7)
+    c = o.project_ic(I.perturbed_vortex) + 0.002 * rng.standard_normal((o.N, 4, o.np))
+    lam = rng.standard_normal(c.shape)
+    assert rel_l2(_host(m.rhs_adjoint(_dev(c), _dev(lam))), o.rhs_vjp(c, lam)) < 1e-12
+    dt = I.fixed_dt(mesh, I.perturbed_vortex, p)
+    assert rel_l2(_host(m.adjoint_step(_dev(c), dt, _dev(lam))), o.ssp_rk3_vjp(c, dt, lam)) < 1e-12
+    m.device_status()
+
+
+def test_adjoint_boundary_and_stages(dgmod, oracle_mod):
+    mesh = I.box_mesh(61, I.BC_WALL, I.BC_STATE)
+    m = dgmod.Mesh.from_mesh(mesh, 2)
+    o = oracle_mod.OracleDG.from_mesh(mesh, 2)
+    xy = o.boundary_points()
+    ub = np.ascontiguousarray(I.steady_vortex(xy[..., 0], xy[..., 1]))
+    o.set_boundary_state(ub)
+    m.set_boundary_state(_dev(ub))
+    rng = np.random.default_rng(8)
+    c = o.project_ic(I.steady_vortex) + 0.002 * rng.standard_normal((o.N, 4, o.np))
+    lam = rng.standard_normal(c.shape)
+    dt = I.fixed_dt(mesh, I.steady_vortex, 2)
+    got = _host(m.adjoint_step(_dev(c), dt, _dev(lam)))
+    assert rel_l2(got, o.ssp_rk3_vjp(c, dt, lam)) < 1e-12
+    import torch
+    d = _dev(c)
+    u1, u2 = torch.empty_like(d), torch.empty_like(d)
+    m.rk_step_stages(d, dt, u1, u2)
+    assert np.array_equal(got, _host(m.adjoint_step_stages(_dev(c), u1, u2, dt, _dev(lam))))
