@@ -158,51 +158,54 @@ k_adj_face(const double *__restrict__ T, const double *__restrict__ G, double *_
            const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const double *__restrict__ bstate,
            int64_t N, int64_t F, double gamma, int *err) {
   constexpr int NF = 3 * NE;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= F * NE) return;
-  const int64_t f = i / NE;
+  const uint32_t i = blockIdx.x * (uint32_t)blockDim.x + threadIdx.x;    // F NE < 2^32 (face_flux_points)
+  if (i >= (uint32_t)(F * NE)) return;
+  const uint32_t f = i / NE;
   const int k = (int)(i - f * NE);
   const FaceConn cn = conn[f];
-  const FaceGeo g = fg[f];
+  const FaceGeo *g = fg + f;
+  const double nx = g->nx, ny = g->ny, hh = half_bits(g->hl);
   const size_t ol = ((size_t)checked(cn.l, N, err) * NF + checked(cn.L, 3, err) * NE + k) * M;
   double ul[M], ur[M], fb[M], gl[M], gr[M];
+  auto get = [](const double *p, double v[M]) {               // 32-byte aligned
+    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  };
+  auto put = [](double *p, const double v[M]) {
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+  };
+  get(T + ol, ul);
+  get(G + ol, gl);
   if (cn.r < 0) {
     // boundary face: F_hat(U_l, U_g(U_l)).  A wall's ghost is the reflection
     // U_g = Rf U_l, Rf = diag(1, I - 2 n n^T, 1) (symmetric), so the trace's
     // cotangent is gl + Rf gr; a prescribed ghost does not depend on U_l.  Only
     // the left element lifts the flux (with -1).
+    ghost_state(cn.r, ul, nx, ny, bstate + ((size_t)f * NE + k) * M, ur);
 #pragma unroll
-    for (int m = 0; m < M; ++m) ul[m] = T[ol + m];
-    ghost_state(cn.r, ul, g.nx, g.ny, bstate + ((size_t)f * NE + k) * M, ur);
-#pragma unroll
-    for (int m = 0; m < M; ++m) fb[m] = -g.hl * G[ol + m];
-    lax_friedrichs_vjp(ul, ur, g.nx, g.ny, gamma, fb, gl, gr);
+    for (int m = 0; m < M; ++m) fb[m] = -hh * gl[m];
+    lax_friedrichs_vjp(ul, ur, nx, ny, gamma, fb, gl, gr);
     if (cn.r == DG_BC_WALL) {
-      const double gn2 = 2.0 * fma(gr[1], g.nx, gr[2] * g.ny);
+      const double gn2 = 2.0 * fma(gr[1], nx, gr[2] * ny);
       gl[0] += gr[0];
-      gl[1] += fma(-gn2, g.nx, gr[1]);
-      gl[2] += fma(-gn2, g.ny, gr[2]);
+      gl[1] += fma(-gn2, nx, gr[1]);
+      gl[2] += fma(-gn2, ny, gr[2]);
       gl[3] += gr[3];
     }
-#pragma unroll
-    for (int m = 0; m < M; ++m) TB[ol + m] = gl[m];
+    put(TB + ol, gl);
     return;
   }
   const size_t orr = ((size_t)checked(cn.r, N, err) * NF + checked(cn.R, 3, err) * NE + (NE - 1 - k)) * M;
+  get(T + orr, ur);
+  get(G + orr, gr);
+  // fhat = l F_hat enters the left element with -1 and the right element with +1
+  // (half of the cotangent: lax_friedrichs_vjp)
 #pragma unroll
-  for (int m = 0; m < M; ++m) {
-    ul[m] = T[ol + m];
-    ur[m] = T[orr + m];
-    // fhat enters the left element with -1 and the right element with +1;
-    // fhat = l * F_hat
-    fb[m] = g.hl * (G[orr + m] - G[ol + m]);
-  }
-  lax_friedrichs_vjp(ul, ur, g.nx, g.ny, gamma, fb, gl, gr);
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    TB[ol + m] = gl[m];
-    TB[orr + m] = gr[m];
-  }
+  for (int m = 0; m < M; ++m) fb[m] = hh * (gr[m] - gl[m]);
+  lax_friedrichs_vjp(ul, ur, nx, ny, gamma, fb, gl, gr);
+  put(TB + ol, gl);
+  put(TB + orr, gr);
 }
 
 template <int P, int NE>

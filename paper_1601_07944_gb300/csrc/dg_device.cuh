@@ -361,21 +361,6 @@ __device__ __forceinline__ void face_flux_points(const double *__restrict__ trac
   if (!ok) atomicOr(err, kErrNonPhysical);
 }
 
-// 1/sqrt(x) for a finite x > 0 in float64: Newton-Raphson refinement of a float32
-// estimate r (rsqrt.approx.ftz.f32 on x rounded to float32), twice
-// r <- r + r (1/2 - (x/2) r^2); the estimate is good to about 2^-22 and each step
-// squares the relative error (dg_self_test checks the result against
-// 1 / sqrt(x): at most 1 ulp apart).  Seven float64 operations.
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  const float xf = f64_to_f32_dev(x);
-  float rf;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(xf));
-  double r = f32_to_f64_dev(rf);
-  const double h = 0.5 * x;
-  r = fma(r, fma(-h * r, r, 0.5), r);
-  return fma(r, fma(-h * r, r, 0.5), r);
-}
-
 // x with the sign of s applied, and 0 where s is zero (d|s|/ds times x with
 // sign(0) = 0), on the bit patterns
 __device__ __forceinline__ double sign_times(double s, double x) {
@@ -386,35 +371,46 @@ __device__ __forceinline__ double sign_times(double s, double x) {
 }
 
 // The quantities of one Euler state that the transposed flux and wave-speed
-// Jacobians share: 1/rho, velocity (u, v), |v|^2, pressure p, E + p, v.n.
+// Jacobians share: 1/rho, velocity (u, v), |v|^2 / 2, P / rho = p / ((gamma-1) rho),
+// enthalpy (E+p) / rho, v.n, and 1/c and the wave speed |v.n| + c.  Twelve float64
+// operations: the reciprocal and the reciprocal square root are formed in integers
+// (which this GPU issues 64 times as fast), halving is an exponent.
 struct EulerSide {
-  double inv, u, v, q2, p, H, vn;
+  double inv, u, v, h2, Pr, Hr, vn, rc, speed;
 };
-__device__ __forceinline__ EulerSide euler_side(const double U[M], double nx, double ny, double g1) {
+__device__ __forceinline__ double half_bits(double x) {         // x / 2 of a normal x or zero
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7FFFFFFF) >= 0x00200000 ? hi - 0x00100000 : hi & (int)0x80000000, __double2loint(x));
+}
+__device__ __forceinline__ EulerSide euler_side(const double U[M], double nx, double ny, double g1, double gg1) {
   EulerSide s;
-  s.inv = recip(U[0]);
+  s.inv = fx::recip_fixed(U[0]);
   s.u = U[1] * s.inv;
   s.v = U[2] * s.inv;
-  s.q2 = fma(s.u, s.u, s.v * s.v);
-  s.p = g1 * fma(-0.5 * U[0], s.q2, U[3]);
-  s.H = U[3] + s.p;
+  s.h2 = half_bits(fma(s.u, s.u, s.v * s.v));
+  const double Er = U[3] * s.inv;
+  s.Pr = Er - s.h2;
+  s.Hr = fma(g1, s.Pr, Er);
   s.vn = fma(s.u, nx, s.v * ny);
+  const double x = gg1 * s.Pr;                                  // c^2 = gamma p / rho
+  s.rc = fx::rsqrt_fixed(x);
+  s.speed = fma(x, s.rc, fabs(s.vn));
   return s;
 }
 
 // out = (d(F(U).n)/dU)^T b for the Euler flux F.n = (rho vn, mx vn + p nx,
 // my vn + p ny, (E+p) vn), using d vn/dU = (-vn, nx, ny, 0)/rho and
 // dp/dU = (gamma-1) (|v|^2/2, -u, -v, 1):
-//   sig = (b1 mx + b2 my + b3 (E+p)) / rho,  tau = (gamma-1) (b1 nx + b2 ny + b3 vn),
-//   out = (-sig vn + tau |v|^2 / 2, b0 nx + b1 vn + sig nx - tau u,
-//          b0 ny + b2 vn + sig ny - tau v, b3 vn + tau).
-__device__ __forceinline__ void flux_jac_t(const double U[M], const EulerSide &s, double nx, double ny, double g1,
+//   sig = b1 u + b2 v + b3 (E+p) / rho,  tau = (gamma-1) (bn + b3 vn),  bn = b1 nx + b2 ny,
+//   out = (tau |v|^2 / 2 - sig vn, (b0 + sig) nx + b1 vn - tau u,
+//          (b0 + sig) ny + b2 vn - tau v, b3 vn + tau).
+__device__ __forceinline__ void flux_jac_t(const EulerSide &s, double nx, double ny, double g1, double bn,
                                            const double b[M], double out[M]) {
-  const double sig = fma(b[1], U[1], fma(b[2], U[2], b[3] * s.H)) * s.inv;
-  const double tau = g1 * fma(b[1], nx, fma(b[2], ny, b[3] * s.vn));
-  out[0] = fma(0.5 * tau, s.q2, -sig * s.vn);
-  out[1] = fma(b[0], nx, fma(b[1], s.vn, fma(sig, nx, -tau * s.u)));
-  out[2] = fma(b[0], ny, fma(b[2], s.vn, fma(sig, ny, -tau * s.v)));
+  const double sig = fma(b[1], s.u, fma(b[2], s.v, b[3] * s.Hr));
+  const double tau = g1 * fma(b[3], s.vn, bn), t = b[0] + sig;
+  out[0] = fma(tau, s.h2, -sig * s.vn);
+  out[1] = fma(t, nx, fma(b[1], s.vn, -tau * s.u));
+  out[2] = fma(t, ny, fma(b[2], s.vn, -tau * s.v));
   out[3] = fma(b[3], s.vn, tau);
 }
 
@@ -441,52 +437,45 @@ __device__ __forceinline__ void flux_jac_t_xy(const double U[M], double gamma, c
   out[3] = fma(bx[3], u, fma(by[3], v, T));
 }
 
-// Wave speed s = |v.n| + c of a state and, when ds is not null, its gradient
-// (d|x|/dx = sign(x), sign(0) = 0):  dc = k (dp - p/rho drho), k = gamma / (2 c rho).
-__device__ __forceinline__ double wave_speed(const EulerSide &s, double gamma, double &rc) {
-  const double x = gamma * s.p * s.inv;          // c^2
-  rc = rsqrt_nr(x);                              // 1/c
-  return fabs(s.vn) + x * rc;
-}
-__device__ __forceinline__ void wave_speed_grad(const EulerSide &s, double rc, double nx, double ny, double gamma,
-                                                double ds[M]) {
-  const double g1 = gamma - 1.0;
-  const double k = (0.5 * gamma) * s.inv * rc;
-  const double kg = k * g1;
-  ds[0] = sign_times(s.vn, -s.vn * s.inv) + k * fma(0.5 * g1, s.q2, -s.p * s.inv);
-  ds[1] = fma(-kg, s.u, sign_times(s.vn, nx * s.inv));
-  ds[2] = fma(-kg, s.v, sign_times(s.vn, ny * s.inv));
-  ds[3] = kg;
-}
-
-// Transposed Lax-Friedrichs Jacobians applied to a cotangent fb:
-//   gl = (dF_hat/dUl)^T fb,  gr = (dF_hat/dUr)^T fb,
-// dF_hat/dUl = A(Ul)/2 + alpha/2 I - (Ur-Ul)/2 (x) d alpha/dUl, and alike for Ur;
+// Transposed Lax-Friedrichs Jacobians applied to a cotangent, given half of it, b:
+//   gl = (dF_hat/dUl)^T 2b,  gr = (dF_hat/dUr)^T 2b,
+// dF_hat/dUl = A(Ul)/2 + alpha/2 I - (Ur-Ul)/2 (x) d alpha/dUl, and alike for Ur, so
+//   gl = A(Ul)^T b + alpha b - ((Ur-Ul).b) d alpha/dUl;
 // d alpha follows the larger wave speed, the left one at a tie (the speeds are
-// compared on their bit patterns: both are >= 0).
-__device__ __forceinline__ void lax_friedrichs_vjp(const double ul[M], const double ur[M], double nx,
-                                                   double ny, double gamma, const double fb[M],
-                                                   double gl[M], double gr[M]) {
-  const double g1 = gamma - 1.0;
-  const EulerSide Sl = euler_side(ul, nx, ny, g1), Sr = euler_side(ur, nx, ny, g1);
-  double rcl, rcr;
-  const double sl = wave_speed(Sl, gamma, rcl), sr = wave_speed(Sr, gamma, rcr);
-  const bool left = __double_as_longlong(sl) >= __double_as_longlong(sr);
-  const double a = left ? sl : sr;
-  double ds[M];
-  wave_speed_grad(left ? Sl : Sr, left ? rcl : rcr, nx, ny, gamma, ds);
-  double jump = (ur[0] - ul[0]) * fb[0];
+// compared on their bit patterns: both are >= 0), with d|x|/dx = sign(x),
+// sign(0) = 0 and dc = k (dp - p/rho drho), k = gamma / (2 c rho):
+//   d alpha/dU = (-+vn/rho + kg (|v|^2/2 - P/rho), +-nx/rho - kg u, +-ny/rho - kg v, kg),
+//   kg = (gamma-1) k, P = p / (gamma-1).
+// About 86 float64 operations.
+__device__ __forceinline__ void lax_friedrichs_vjp(const double ul[M], const double ur[M], double nx, double ny,
+                                                   double gamma, const double b[M], double gl[M], double gr[M]) {
+  const double g1 = gamma - 1.0, gg1 = gamma * g1;
+  const EulerSide Sl = euler_side(ul, nx, ny, g1, gg1), Sr = euler_side(ur, nx, ny, g1, gg1);
+  const bool left = __double_as_longlong(Sl.speed) >= __double_as_longlong(Sr.speed);
+  const double a = left ? Sl.speed : Sr.speed;
+  double jump = (ur[0] - ul[0]) * b[0];
 #pragma unroll
-  for (int m = 1; m < M; ++m) jump = fma(ur[m] - ul[m], fb[m], jump);
+  for (int m = 1; m < M; ++m) jump = fma(ur[m] - ul[m], b[m], jump);
+  const double bn = fma(b[1], nx, b[2] * ny);
   double jl[M], jr[M];
-  flux_jac_t(ul, Sl, nx, ny, g1, fb, jl);
-  flux_jac_t(ur, Sr, nx, ny, g1, fb, jr);
-  const double ha = 0.5 * a, hj = 0.5 * jump;
+  flux_jac_t(Sl, nx, ny, g1, bn, b, jl);
+  flux_jac_t(Sr, nx, ny, g1, bn, b, jr);
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    const double t = hj * ds[m];
-    gl[m] = fma(0.5, jl[m], fma(ha, fb[m], left ? -t : 0.0));
-    gr[m] = fma(0.5, jr[m], fma(-ha, fb[m], left ? 0.0 : -t));
+    gl[m] = fma(a, b[m], jl[m]);
+    gr[m] = fma(-a, b[m], jr[m]);
+  }
+  const double inv = left ? Sl.inv : Sr.inv, u = left ? Sl.u : Sr.u, v = left ? Sl.v : Sr.v;
+  const double vn = left ? Sl.vn : Sr.vn;
+  const double kg = half_bits(gg1) * inv * (left ? Sl.rc : Sr.rc);
+  const double si = sign_times(vn, inv);
+  const double ds[M] = {fma(kg, left ? Sl.h2 - Sl.Pr : Sr.h2 - Sr.Pr, -vn * si), fma(-kg, u, nx * si),
+                        fma(-kg, v, ny * si), kg};
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const double t = fma(-jump, ds[m], left ? gl[m] : gr[m]);
+    if (left) gl[m] = t;
+    else gr[m] = t;
   }
 }
 

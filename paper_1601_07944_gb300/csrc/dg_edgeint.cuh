@@ -186,6 +186,30 @@ DG_HD double recip_fixed(double x) {
   return of_bits(r);
 }
 
+// 1/sqrt(x) as a float64, rounded to nearest (to 2^-58 before that), for a positive
+// normal x; NaN for any other.  x = v 4^k with v in [2^60, 2^62); a float32 estimate
+// y (23 bits) of 2^53 / sqrt(v) and its residual e = 1 - v y^2 / 2^106, exact to
+// 2^-61, give y (1 + e/2 + 3 e^2 / 8); the next term is below 2^-64.
+DG_HD double rsqrt_fixed(double x) {
+  const long long b = bits_of(x);
+  const int be = (int)(b >> 52);                                // biased exponent (negative: x < 0)
+  const int odd = ~be & 1;                                      // be - 1083 odd
+  const long long v = ((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << (8 + odd);
+  const int k = (be - 1083 - odd) >> 1;
+  const Half2x31 c = cut(v);
+  const int y = to_int(rsqrt32((float)c.h) * 194368031998.42758f);              // 2^37.5
+  const long long t = ((long long)c.h * y << 8) + (((long long)c.l * y) >> 23);   // v y / 2^23
+  const Half2x31 tc = cut(t);
+  const long long u = (1ll << 52) - (long long)tc.h * y;
+  const long long e = (long long)((unsigned long long)u << 31) - (long long)tc.l * y;   // e 2^83
+  const int eh = (int)(e >> 32);
+  const long long z = (long long)y * eh + (long long)(((unsigned long long)(uint32_t)y * (uint32_t)e) >> 32);   // y e 2^51
+  const long long q = ((long long)(int)(z >> 31) * eh * 3) >> 36;
+  const long long r = ((long long)y << 38) + (z >> 14) + q;                     // 2^91 / sqrt(v)
+  const long long out = ((r + 128) >> 8) + ((long long)(991 - k) << 52);
+  return of_bits((unsigned)(be - 1) >= 2046u ? 0x7FF8000000000000ll : out);
+}
+
 // sqrt(v) 2^30 for v in [2^58, 2^62): in [2^59, 2^61)
 DG_HD long long sqrt_fixed(long long v) {
   const float f = (float)(int)(v >> 31);                        // v 2^-31, 24 bits
@@ -205,9 +229,9 @@ DG_HD long long sqrt_fixed(long long v) {
 
 }  // namespace fx
 
-inline FaceFix face_fix(double sx, double sy, double hk) {
-  auto ex = [](double x) { return (int)((fx::bits_of(x) >> 52) & 0x7FF); };
-  const int es = ex(sx) > ex(sy) ? ex(sx) : ex(sy), ek = ex(hk);
+DG_HD int exponent_of(double x) { return (int)((fx::bits_of(x) >> 52) & 0x7FF); }
+DG_HD FaceFix face_fix(double sx, double sy, double hk) {
+  const int ex = exponent_of(sx), ey = exponent_of(sy), es = ex > ey ? ex : ey, ek = exponent_of(hk);
   const bool in = es > 723 && es < 1323 && ek > 723 && ek < 1323 && hk > 0.0;
   return FaceFix{fx::fixed_of(sx, es), fx::fixed_of(sy, es), fx::fixed_of(hk, ek) * 2, in ? es : -1, ek};
 }

@@ -622,8 +622,6 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       elem_face[3 * f + qf] = 2 * fi + 1;
     }
   const int64_t F = (int64_t)conn.size();
-  std::vector<FaceFix> ffix(F);
-  for (int64_t i = 0; i < F; ++i) ffix[i] = face_fix(fgeo[i].sx, fgeo[i].sy, fgeo[i].hk);
 
   // --- tables ----------------------------------------------------------------
   const int np = (p + 1) * (p + 2) / 2, nd = p + 1, nf = 3 * ne;
@@ -814,7 +812,7 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       (ce = cudaMemcpy(m->elem_face, elem_face.data(), sizeof(int32_t) * N * 3, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->face_conn, conn.data(), sizeof(FaceConn) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemcpy(m->face_geo, fgeo.data(), sizeof(FaceGeo) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (ce = cudaMemcpy(m->face_fix, ffix.data(), sizeof(FaceFix) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (ce = (cudaError_t)dg::launch_face_fix(m)) != cudaSuccess ||
       (ce = cudaMemcpy(m->table_block, tb.data(), sizeof(double) * off, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = cudaMemset(m->err_flag, 0, sizeof(int))) != cudaSuccess ||
       (ce = (cudaError_t)dg::tc_tables(m)) != cudaSuccess ||

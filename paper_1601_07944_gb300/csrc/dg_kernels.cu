@@ -94,6 +94,12 @@ k_face(const double *__restrict__ trace, double *__restrict__ fhat, const FaceCo
   face_flux_points<NE>(trace, fhat, conn, fg, ff, bstate, N, F, gf, err, blockIdx.x, gridDim.x);
 }
 
+__global__ void __launch_bounds__(kThreads)
+k_face_fix(const FaceGeo *__restrict__ fg, FaceFix *__restrict__ ff, int64_t F) {
+  const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (f < F) ff[f] = face_fix(fg[f].sx, fg[f].sy, fg[f].hk);
+}
+
 // ---------------------------------------------------------------------------
 // projection of point data and volume point coordinates
 // ---------------------------------------------------------------------------
@@ -408,6 +414,11 @@ int launch_limit(const dg_mesh *m, double *c, double *trace, int have_traces, vo
     k_limit_p1<false><<<resident_grid(m, (const void *)k_limit_p1<false>, kThreads, m->N * M, &per_sm[0]), kThreads,
                          0, s>>>(c, trace, m->elem_nbr, m->tab.EPa, m->tab.EChiM1, m->tab.EChi, m->phi1, m->N,
                                  m->err_flag);
+  return (int)cudaGetLastError();
+}
+
+int launch_face_fix(dg_mesh *m) {
+  k_face_fix<<<(int)((m->F + kThreads - 1) / kThreads), kThreads>>>(m->face_geo, m->face_fix, m->F);
   return (int)cudaGetLastError();
 }
 

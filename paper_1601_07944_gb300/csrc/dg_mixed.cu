@@ -152,7 +152,7 @@ __global__ void k_convert_check(int n, unsigned long long *bad) {
     if (d > 1 || d3 > 1 || di > 1) atomicAdd(bad + 2, 1ull);
     const long long qs = __double_as_longlong(sqrt(ax)), rs = __double_as_longlong(sqrt_nr(ax));
     const long long ds = qs > rs ? qs - rs : rs - qs;
-    const long long qr = __double_as_longlong(1.0 / sqrt(ax)), rr = __double_as_longlong(rsqrt_nr(ax));
+    const long long qr = __double_as_longlong(1.0 / sqrt(ax)), rr = __double_as_longlong(fx::rsqrt_fixed(ax));
     const long long dr = qr > rr ? qr - rr : rr - qr;
     if (ds > 1 || dr > 2) atomicAdd(bad + 3, 1ull);
   }
