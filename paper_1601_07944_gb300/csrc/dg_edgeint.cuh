@@ -117,7 +117,16 @@ DG_HD long long mul(Half2x31 a, Half2x31 b) {
   const long long c = (long long)a.h * b.l + (long long)a.l * b.h;
   return (long long)a.h * b.h + (c >> 31);
 }
-DG_HD long long sqr(Half2x31 a) { return (long long)a.h * a.h + (((long long)a.h * a.l) >> 30); }
+// the same for a b4 / 2^64 of unsigned numbers, the second taken times four: on the
+// device four multiplies, where the halves above take eight instructions of the
+// busier pipe
+DG_HD unsigned long long umul(unsigned long long a, unsigned long long b4) {
+#ifdef __CUDA_ARCH__
+  return __umul64hi(a, b4);
+#else
+  return (unsigned long long)(((unsigned __int128)a * b4) >> 64);
+#endif
+}
 DG_HD long long shr(long long x, int d) { return x >> (d < 63 ? d : 63); }
 
 // the same, rounded to nearest (a small negative x gives 0, not -1)
@@ -128,7 +137,7 @@ DG_HD long long shr_rn(long long x, int d) {
 
 // x 2^(1083 - e), truncated toward zero, for a float64 x of biased exponent at most
 // e (e >= 63, so that a zero comes out as 0): below 2^61
-DG_HD long long fixed_of(double x, int e) {
+DG_HD long long fixed_of(double x, int e, unsigned long long *magnitude = nullptr) {
   const long long b = bits_of(x);
   const int hi = (int)(b >> 32);
   const int own = (hi >> 20) & 0x7FF;
@@ -136,6 +145,7 @@ DG_HD long long fixed_of(double x, int e) {
   const unsigned long long m = ((unsigned long long)((mh << 8) | (l >> 24)) << 32) | (l << 8);
   const int d = e - own;
   const long long v = (long long)(m >> (d < 63 ? d : 63));
+  if (magnitude) *magnitude = (unsigned long long)v;
   const long long s = (long long)(hi >> 31);
   return (v ^ s) - s;
 }
@@ -222,7 +232,7 @@ DG_HD long long sqrt_fixed(long long v) {
   const int t = to_int((float)(int)(e >> 11) * (h * 8589934592.0f));        // e / (2 b) 2^22
   const long long c1 = ((long long)b << 30) + (long long)t * 256;
   // the rest, from c1^2 / 2^62 against v / 4
-  const int e1 = (int)((v >> 2) - sqr(cut(c1)));
+  const int e1 = (int)((v >> 2) - (long long)umul((unsigned long long)c1, (unsigned long long)c1 * 4));
   const int t1 = to_int((float)e1 * (h * 4294967296.0f));
   return c1 + t1;
 }
@@ -262,7 +272,6 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   if (!ok) return false;
   const Half2x31 Sx = cut(g.sx), Sy = cut(g.sy);
   const Half2x31 G1 = cut(g1);
-  const Half2x31 HK = cut(g.hk);
   long long w[2], Pf[2], c[2];
   int xc[2];
 #pragma unroll
@@ -271,18 +280,20 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
     const int re = s ? rR : rL;
     const long long y = recip_mantissa(u[0]);                   // 1/rho = y 2^(961 - re)
     const long long yc = y < (1ll << 62) ? y : (1ll << 62) - 1;
-    const Half2x31 Y = cut(yc), I = cut(yc >> (1 + re - r0));   // 1/rho = I 2^(962 - r0)
-    const Half2x31 Mx = cut(fixed_of(u[1], em)), My = cut(fixed_of(u[2], em));
+    const long long I = yc >> (1 + re - r0);                    // 1/rho = I 2^(962 - r0)
+    unsigned long long ax, ay;
+    const Half2x31 Mx = cut(fixed_of(u[1], em, &ax)), My = cut(fixed_of(u[2], em, &ay));
     const long long mn = mul(Mx, Sx) + mul(My, Sy);
-    w[s] = mul(cut(mn), I);                                     // X = em + es - r0 - 1080
-    const long long q = sqr(Mx) + sqr(My);
-    const long long K = mul(cut(q), I);                         // |m|^2 / rho, X = 2 em - r0 - 1080
+    const long long sn = mn >> 63;                              // X = em + es - r0 - 1080
+    w[s] = ((long long)umul((unsigned long long)((mn ^ sn) - sn), (unsigned long long)I * 4) ^ sn) - sn;
+    const unsigned long long q = umul(ax, ax * 4) + umul(ay, ay * 4);
+    const long long K = (long long)umul(q, (unsigned long long)I * 4);   // |m|^2 / rho, X = 2 em - r0 - 1080
     Pf[s] = (fixed_of(u[3], eE + 6) - shr(K, dK)) * 64;         // p / (gamma - 1), X = eE - 1083
     ok &= Pf[s] > 0;
     const int z = clz64((unsigned long long)Pf[s]) - 2;         // Pf 2^z in [2^61, 2^62)
     const long long Pn = (long long)((unsigned long long)Pf[s] << (z & 63));
     // c^2 = hk P / rho, h^2 folded in: X = eE - 1083 - z - re + ek + 1
-    long long c2 = mul(cut(mul(cut(Pn), Y)), HK);
+    long long c2 = (long long)umul(umul((unsigned long long)Pn, (unsigned long long)yc * 4), (unsigned long long)g.hk * 4);
     int x2 = eE - 1082 - z - re + g.ek;
     c2 = (x2 & 1) ? c2 >> 1 : c2;
     x2 += x2 & 1;
@@ -298,7 +309,7 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   const long long la = al > ar ? al : ar;
   const double wa = to_double(wl + la, xa), wb = to_double(wr - la, xa);
   // (gamma - 1) (P_l + P_r) and (gamma - 1) (P_l w_l + P_r w_r)
-  const double ps = to_double(mul(cut((Pf[0] + Pf[1]) >> 1), G1), eE - 1083 + 1 + 62 + eg - 1083);
+  const double ps = to_double((long long)umul((unsigned long long)(Pf[0] + Pf[1]) >> 1, (unsigned long long)g1 * 4), eE - 1083 + 1 + 62 + eg - 1083);
   const long long pw = mul(cut(Pf[0]), cut(w[0])) + mul(cut(Pf[1]), cut(w[1]));
   const double H = to_double(mul(cut(pw), G1), eE - 1083 + 62 + xw + 62 + eg - 1083);
 #ifdef __CUDA_ARCH__

@@ -86,8 +86,12 @@ k_traces(const double *__restrict__ c, double *__restrict__ trace, const double 
 // ---------------------------------------------------------------------------
 // edge flux: fhat[f][k][m] = l_f * F_hat(U_l(r_{L,k}), U_r(r_{R,NE-1-k}), n_f)
 // ---------------------------------------------------------------------------
+// One item a thread in blocks of 128: a resident grid's equal slices leave it partly
+// idle for the last of a few turns (256 x 256, p = 3: 5.05 items a thread, 24 of 32
+// warps active on average).
+constexpr int kFaceThreads = 128;
 template <int NE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kFaceThreads)
 k_face(const double *__restrict__ trace, double *__restrict__ fhat, const FaceConn *__restrict__ conn,
        const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff, const double *__restrict__ bstate, int64_t N,
        int64_t F, GammaFix gf, int *err) {
@@ -425,13 +429,9 @@ int launch_face_fix(dg_mesh *m) {
 int launch_face_flux(const dg_mesh *m, const double *trace, double *fhat, void *stream) {
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = m->F * m->ne;
-#define FACE(NE)                                                                                        \
-  do {                                                                                                  \
-    static int per_sm = 0;                                                                              \
-    k_face<NE><<<resident_grid(m, (const void *)k_face<NE>, kThreads, n, &per_sm), kThreads, 0, s>>>(   \
-        trace, fhat, m->face_conn, m->face_geo, m->face_fix, m->bstate, m->N, m->F, gamma_fix(m->gamma),   \
-        m->err_flag);                                                                                   \
-  } while (0)
+#define FACE(NE)                                                                                                 \
+  k_face<NE><<<(unsigned)((n + kFaceThreads - 1) / kFaceThreads), kFaceThreads, 0, s>>>(                         \
+      trace, fhat, m->face_conn, m->face_geo, m->face_fix, m->bstate, m->N, m->F, gamma_fix(m->gamma), m->err_flag)
   switch (m->ne) {
     case 2: FACE(2); break;
     case 3: FACE(3); break;

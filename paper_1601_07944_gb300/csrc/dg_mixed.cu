@@ -42,16 +42,16 @@ namespace {
 // BND: the launch covers the boundary faces [f0, f1) = [0, Fb) (a ghost state on
 // the right, Algorithm 2); otherwise the interior faces [Fb, F), in a separate
 // instantiation so that the common case carries no boundary code.
+constexpr int kMixedFaceThreads = 64;
 template <int NE, bool BND>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(kMixedFaceThreads, 768 / kMixedFaceThreads)
 k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *__restrict__ fmean,
              const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff,
              const double *__restrict__ Lf, const double *__restrict__ bstate, int np, int64_t N, int64_t f0,
              int64_t f1, GammaFix gf, int *err) {
   constexpr int NF = 3 * NE;
   bool ok = true;
-  // the grid is what is resident at once; block b takes the b-th of gridDim.x
-  // equal slices of the edges
+  // block b takes the b-th of gridDim.x equal slices of the edges
   const int64_t F = f1 - f0;
   const int64_t lo = f0 + F * blockIdx.x / gridDim.x, hi = f0 + F * (blockIdx.x + 1) / gridDim.x;
   for (int64_t f = lo + threadIdx.x; f < hi; f += blockDim.x) {
@@ -189,16 +189,17 @@ MixedBuffers mixed_buffers(const dg_mesh *m, double *trace, double *fhat) {
 
 int launch_face_flux_mixed(const dg_mesh *m, const MixedBuffers &b, void *stream) {
   cudaStream_t s = (cudaStream_t)stream;
+  // an edge a thread, not a resident grid (k_face)
+  auto grid = [](int64_t n) { return (unsigned)((n + kMixedFaceThreads - 1) / kMixedFaceThreads); };
+  const int64_t inner = m->F - m->Fb;
 #define FACE(NE)                                                                                          \
   do {                                                                                                    \
-    static int per_sm = 0, per_sm_b = 0;                                                                  \
-    k_face_mixed<NE, false><<<resident_grid(m, (const void *)k_face_mixed<NE, false>, 256, m->F - m->Fb,   \
-                                            &per_sm), 256, 0, s>>>(                                       \
-        b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N,  \
-        m->Fb, m->F, gamma_fix(m->gamma), m->err_flag);                                                   \
+    if (inner > 0)                                                                                        \
+      k_face_mixed<NE, false><<<grid(inner), kMixedFaceThreads, 0, s>>>(                                  \
+          b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N, \
+          m->Fb, m->F, gamma_fix(m->gamma), m->err_flag);                                                 \
     if (m->Fb > 0)                                                                                        \
-      k_face_mixed<NE, true><<<resident_grid(m, (const void *)k_face_mixed<NE, true>, 256, m->Fb,         \
-                                             &per_sm_b), 256, 0, s>>>(                                    \
+      k_face_mixed<NE, true><<<grid(m->Fb), kMixedFaceThreads, 0, s>>>(                                   \
           b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N, \
           0, m->Fb, gamma_fix(m->gamma), m->err_flag);                                                    \
   } while (0)
