@@ -214,7 +214,6 @@ namespace dg {
 int launch_traces(const dg_mesh *m, const double *c, double *trace, void *stream, double *copy = nullptr);
 int launch_face_flux(const dg_mesh *m, const double *trace, double *fhat, void *stream);
 int launch_face_fix(dg_mesh *m);       // m->face_fix from m->face_geo (mesh creation)
-int resident_grid(const dg_mesh *m, const void *kernel, int threads, int64_t n, int *per_sm);
 // out = mode==0 ? R(c) : the stage update su (and su.out2);  trace_out may be null.
 // Elements [e0, e1) only (e1 < 0: all; the same bits per element either way).
 int launch_element(const dg_mesh *m, const double *c, const double *u0, double *out,

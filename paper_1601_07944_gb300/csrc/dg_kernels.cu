@@ -352,8 +352,9 @@ __global__ void __launch_bounds__(kThreads) k_fma_probe(int iters, double *out) 
 // Barth-Jespersen limiter for p = 1 (Section 4.3.5), in place on c: the items of
 // limit_p1_items (dg_limiter.cuh) over the grid.
 // ---------------------------------------------------------------------------
+constexpr int kLimitThreads = 128;
 template <bool HAVE_TRACES>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kLimitThreads)
 k_limit_p1(double *c, double *__restrict__ trace, const int32_t *__restrict__ elem_nbr,
            const double *__restrict__ EPa, const double *__restrict__ EChiM1, const double *__restrict__ EChi,
            double phi1, int64_t N, int *err) {
@@ -389,35 +390,17 @@ int launch_traces(const dg_mesh *m, const double *c, double *trace, void *stream
   return (int)cudaErrorInvalidValue;
 }
 
-// blocks of `threads` threads needed for n items, at most what is resident on
-// the GPU at once (a grid-stride kernel covers the rest); per_sm is the kernel's
-// resident blocks per SM (0: ask the occupancy calculator)
-int resident_grid(const dg_mesh *m, const void *kernel, int threads, int64_t n, int *per_sm) {
-  if (*per_sm == 0) {
-    int v = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, threads, 0) != cudaSuccess || v < 1) {
-      cudaGetLastError();
-      v = 1;
-    }
-    *per_sm = v;
-  }
-  const int64_t need = (n + threads - 1) / threads, cap = (int64_t)m->num_sms * *per_sm;
-  return (int)(need < cap ? (need > 0 ? need : 1) : cap);
-}
-
 int launch_limit(const dg_mesh *m, double *c, double *trace, int have_traces, void *stream) {
   if (m->p != 1 || m->ne != 2) return (int)cudaErrorInvalidValue;
   if (have_traces && !trace) return (int)cudaErrorInvalidValue;
-  static int per_sm[2] = {0, 0};
   cudaStream_t s = (cudaStream_t)stream;
+  const unsigned grid = (unsigned)((m->N * M + kLimitThreads - 1) / kLimitThreads);
   if (have_traces)
-    k_limit_p1<true><<<resident_grid(m, (const void *)k_limit_p1<true>, kThreads, m->N * M, &per_sm[1]), kThreads,
-                        0, s>>>(c, trace, m->elem_nbr, m->tab.EPa, m->tab.EChiM1, m->tab.EChi, m->phi1, m->N,
-                                m->err_flag);
+    k_limit_p1<true><<<grid, kLimitThreads, 0, s>>>(c, trace, m->elem_nbr, m->tab.EPa, m->tab.EChiM1, m->tab.EChi,
+                                                   m->phi1, m->N, m->err_flag);
   else
-    k_limit_p1<false><<<resident_grid(m, (const void *)k_limit_p1<false>, kThreads, m->N * M, &per_sm[0]), kThreads,
-                         0, s>>>(c, trace, m->elem_nbr, m->tab.EPa, m->tab.EChiM1, m->tab.EChi, m->phi1, m->N,
-                                 m->err_flag);
+    k_limit_p1<false><<<grid, kLimitThreads, 0, s>>>(c, trace, m->elem_nbr, m->tab.EPa, m->tab.EChiM1, m->tab.EChi,
+                                                    m->phi1, m->N, m->err_flag);
   return (int)cudaGetLastError();
 }
 

@@ -127,10 +127,10 @@ __device__ __forceinline__ void limit_p1_items(double *c, double *__restrict__ t
       dbest = below ? dneg : dbest;
     }
     if (nbest < dbest) {
-      // alpha = nbest / dbest by the Newton-refined reciprocal (within 1.5 ulp of
+      // alpha = nbest / dbest by a reciprocal formed in integers (within 1.5 ulp of
       // the quotient); the traces of the scaled coefficients by the same sums
       // every kernel uses, so that they agree bit for bit with k_traces'
-      const double alpha = bits_value(nbest) * recip(bits_value(dbest));
+      const double alpha = bits_value(nbest) * fx::recip_fixed(bits_value(dbest));
       cj[1] *= alpha;
       cj[2] *= alpha;
       ce[1] = cj[1];

@@ -164,8 +164,7 @@ __device__ __forceinline__ uint32_t pack_digit(uint32_t a, uint32_t b, uint32_t 
 }
 
 // eight values -> four columns of each digit plane of this thread's TMEM lane
-__device__ __forceinline__ void store_digits8(uint32_t tA, int ca, const double *v, int E) {
-  uint32_t w[kDigits][4];
+__device__ __forceinline__ void make_digits8(uint32_t w[kDigits][4], const double *v, int E) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     uint32_t al, ah, bl, bh;
@@ -179,6 +178,10 @@ __device__ __forceinline__ void store_digits8(uint32_t tA, int ca, const double 
     w[4][c] = pack_digit(al >> 10, bl >> 10, MK);
     w[5][c] = pack_digit(al, bl, MK);
   }
+}
+__device__ __forceinline__ void store_digits8(uint32_t tA, int ca, const double *v, int E) {
+  uint32_t w[kDigits][4];
+  make_digits8(w, v, E);
 #pragma unroll
   for (int i = 0; i < kDigits; ++i) tc::st4(tA + (uint32_t)(i * ca), w[i]);
 }
@@ -543,7 +546,6 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       double uv[NPH];
 #pragma unroll
       for (int b = 0; b < T::NB2; ++b) {
-        if (b > 0) mma_wait();                               // the previous batch has read its operand
 #pragma unroll
         for (int s = 0; s < T::KC; s += 8) {
           double x[8];
@@ -552,7 +554,11 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
             const int k = b * T::KC + s + i;
             x[i] = k < NQ ? g[k * M * LD] : (k < T::KH ? fl[k - NQ] : 0.0);
           }
-          store_digits8(tA + (uint32_t)((h * T::KC + s) / 2), T::CA, x, E);
+          uint32_t w[kDigits][4];
+          make_digits8(w, x, E);
+          if (b > 0 && s == 0) mma_wait();                   // the previous batch has read its operand
+#pragma unroll
+          for (int i = 0; i < kDigits; ++i) tc::st4(tA + (uint32_t)((h * T::KC + s) / 2 + i * T::CA), w[i]);
         }
         if (!operands_ready()) return false;
         if (tid == 0) {
