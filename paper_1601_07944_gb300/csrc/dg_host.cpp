@@ -1314,13 +1314,13 @@ static dg_status adjoint_buffers(dg_mesh *m, const char *who) {
     m->adj_doubles = 0;
     cudaError_t e = cudaMalloc(&m->adj_buf, sizeof(double) * need);
     if (e != cudaSuccess) { cudaGetLastError(); return fail(DG_ENOMEM, "%s: cudaMalloc", who); }
-    m->adj_doubles = need;
     if (!m->adj_split_img && (e = (cudaError_t)dg::adj_split_tables(m)) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(m->adj_split_img);
       m->adj_split_img = nullptr;
-      return fail(DG_ECUDA, "%s: tables: %s", who, cudaGetErrorString(e));
+      return fail(e == cudaErrorMemoryAllocation ? DG_ENOMEM : DG_ECUDA, "%s: tables: %s", who, cudaGetErrorString(e));
     }
+    m->adj_doubles = need;             // only now: a failed call leaves none of both behind
   }
   return DG_OK;
 }
