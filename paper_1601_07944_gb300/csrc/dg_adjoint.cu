@@ -27,7 +27,8 @@
  * every contraction with a basis table is the transpose, in reverse order, of a
  * factorised forward contraction with the same table (the collapsed grid is a
  * tensor grid and phi_j(alpha, beta) = P_a(alpha) chi_j(beta)).  The direct
- * kernels above serve the symmetric rules.
+ * kernels above serve the symmetric rules.  At p <= 3 the element pieces of large
+ * meshes run on the tensor cores instead (dg_adj_split.cu, both rules).
  */
 #include <cuda_runtime.h>
 
@@ -152,6 +153,10 @@ k_adj_element(const double *__restrict__ u, const double *__restrict__ lam, doub
   }
 }
 
+// One (edge, point) a thread.  The float64 pipe bounds it: the transposed flux is 86
+// operations (lax_friedrichs_vjp; 141 with separate Jacobians per side and Newton
+// roots), and the narrow pipe takes two lanes a clock (131,072 elements, p = 2: 160
+// -> 110 us).
 template <int NE>
 __global__ void __launch_bounds__(kThreads)
 k_adj_face(const double *__restrict__ T, const double *__restrict__ G, double *__restrict__ TB,

@@ -14,10 +14,9 @@
  * mul(a, b) = a b / 2^62, from 31-bit halves.  Both sides share the exponent of
  * the momenta, of the energies and of w, so that sums need no alignment.
  *
- * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 25 us
- * (p = 1), 66 -> 34 (p = 2), 87 -> 41 (p = 3), 124 -> 59 (p = 5); k_face_mixed 88 ->
- * 53 us (p = 3), 403 -> 204 us (512 x 512, p = 4).  About 900 instructions a point,
- * the integer pipe 53 % busy, the float64 pipe 32 %.  Against 113-bit arithmetic the
+ * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 20 us
+ * (p = 1), 66 -> 29 (p = 2), 87 -> 37 (p = 3), 105 -> 45 (p = 4), 124 -> 54 (p = 5);
+ * k_face_mixed 88 -> 48 us (p = 3), 403 -> 185 us (512 x 512, p = 4).  Against 113-bit arithmetic the
  * error is 0.75-1.0 of the float64 form's (rms) over still, slow, supersonic and
  * discontinuous states.
  *

@@ -5,7 +5,9 @@
  * of the three edge fluxes (Algorithms 2-3), the 1/det J
  * scaling (Eq. 2ddg0), the Runge-Kutta stage update (with, for the classical
  * RK4, the running sum of its stages as a second output) and the next stage's
- * edge traces, for one tile of elements per CTA.
+ * edge traces, for one tile of elements per CTA; and the fused stepper of small
+ * meshes (k_rk_small), whose phases are this kernel's.  Larger meshes take
+ * k_element_split (dg_split.cuh).
  */
 #include <cuda_runtime.h>
 
@@ -822,7 +824,7 @@ int run_element_sf(const dg_mesh *m, const double *c, const double *u0, double *
 // behind the one after the edge fluxes.  (Cycles of a stage, p = 4, 800 elements:
 // 52,500 with whole barriers and the tile read back from memory at each stage, of
 // which 11,500 the barriers, 5,000 the loads and 11,000 the update that waited for
-// its operands.)
+// its operands; 33,900 now.  p = 1, 512 elements: 30,000 -> 17,800.)
 // ---------------------------------------------------------------------------
 constexpr uint64_t kGridWaitNs = 2000000000ull;    // 2 s per barrier before giving up
 

@@ -1,6 +1,6 @@
 /*
  * dg_tcgen05.cuh -- the small set of Blackwell (sm_100a/sm_103a) tensor-core
- * primitives the mixed-precision kernels use, as inline PTX:
+ * primitives the mixed-precision and the split-product kernels use, as inline PTX:
  *
  *   tcgen05.alloc / dealloc        tensor-memory (TMEM) columns for the accumulator
  *   tcgen05.mma.cta_group::1.kind::tf32
@@ -8,6 +8,8 @@
  *                                  shared memory, D in TMEM, FP32 accumulation
  *   tcgen05.mma ... [a-tmem]       the same with A read from TMEM (lane = row of
  *                                  A, one column per TF32 element along K)
+ *   tcgen05.mma ... kind::f16      D[128 x N] (+)= A[128 x 16] B[16 x N], A in TMEM (two
+ *                                  f16 per column), B in shared memory (kmaj16, desc16)
  *   tcgen05.commit -> mbarrier     completion of the issued MMAs
  *   tcgen05.ld.32x32b              TMEM -> registers (each warp reads its own
  *                                  32-lane quarter; lane = accumulator row)
