@@ -53,66 +53,27 @@ WORKLOAD = dict(name="isentropic vortex, 256x256 jittered periodic triangle mesh
                 n=256, p=3, ne=0, cfl=0.3)
 
 
-def flops_element_per_elem(p: int, ne: int) -> float:
-    """Float64 flops of one element-kernel launch per element, for the algorithm
-    the kernel executes (sum factorisation on the collapsed volume grid and on
-    the edges), counting an FMA as 2 flops and a multiply or add as 1:
-      W = chi c                          2 N_p (p+1) 4
-      U = P W (the a = 0 term, P_0 = 1, is a copy)
-                                         2 (p+1)^2 p 4;
-        p >= 3: on the mirror pairs of the Gauss-Legendre nodes, the sums
-        over the even and the odd a and their sum and difference, and for p
-        even the middle node alpha = 0 (P_a(0) = 0 for odd a)
-                                         (p+1) h 4 (2 p + 2) [+ (p+1) 4 p]
-      per volume point: 1/rho (4 FMA Newton steps), pressure, the Euler flux
-      along row 1 of J^tau (H_beta = G_s) and along row 0 + (1+alpha)/2 row 1
-      (H_alpha = G_r + (1+alpha)/2 G_s)  38
-      the directions of H_alpha (2 FMAs each): once per alpha node and element
-      for p >= 3                         4 (p+1); p <= 2: 4 per point
-      Xa, Xb (Xa(0, .) = 0 without arithmetic, P_0' = 0); at p = 2-4 folded on
-      the mirror pairs of the Gauss-Legendre nodes: per (ib, variable) 4 h
-      additions (h = floor((p+1)/2) pairs; at p >= 3 formed in the point phase)
-      and T = (2p+1) h (+ p+1 for p even, the middle node) products
-                                         (p+1) 4 (2 T + 4 h);
-      p = 1: 2 (p+1)^2 (2p+1) 4; p = 5 (every a, on the pair sums and
-      differences): 4 (p+1)^2 h 4 + 16 h (p+1)
-      V = chiA Xa + dchiB Xb (modes with a = 0: the Xb term only)
-                                         (4 (N_p - p - 1) + 2 (p+1)) (p+1) 4
-      lift sums per variable (face 0: omega P_a; faces 1, 2: F1 +/- F2)
-                                         (2 (p+1) n_e + 2 n_e) 4
-      lift per mode                      2 (1 + n_e) N_p 4
-      stage update                       5 N_p 4
-      next traces (face 0 from Z_a = sum_b chi_ab(-1) c_ab, then Z_0 +
-      sum_{a>=1} P_a Z_a; faces 1, 2 from the sums over the modes of even and of
-      odd first index, the constant mode's term chi_00 c_00 formed once)
-                                         (2 N_p + 1 + n_e (2 p + 2 N_p)) 4"""
+def fp64_split_per_elem(p: int, ne: int, nq: int):
+    """(flops, instructions) of the float64 pipe in one launch of the float64
+    element kernel of large meshes (k_element_split) per element, averaged over the
+    three SSP-RK3 stages; an FMA is two flops, and takes an issue slot like a
+    multiply or an add.  The contractions run as integer digit products on the
+    tensor cores and take none; what is left:
+      flux at a point      the reciprocal, p <= 3: 3 FMAs (further up in integers);
+                           |m|^2 and P 3 instructions, 5 flops; E + p 1, 2; along
+                           each of two directions 8, 11
+      stage update         per coefficient 1 FMA in the first stage, a multiply and
+                           2 FMAs in the others
+      edge traces, p = 1   per row and edge point: Z_a and chi_00 c_00 4 (7), then
+                           T_0 1 (2), E and O 2 (4), E +- O 2 (2)"""
     NP = (p + 1) * (p + 2) // 2
-    ND = p + 1
-    h = ND // 2
-    if 2 <= p <= 4:
-        T = (2 * ND - 1) * h + (ND if ND % 2 else 0)
-        x_phase = ND * 4 * (2 * T + 4 * h)
-    elif p == 1:
-        x_phase = 2 * ND * ND * (2 * ND - 1) * 4
-    else:
-        x_phase = 4 * ND * ND * h * 4 + 16 * h * ND
-    if p >= 3:
-        u_phase = ND * h * 4 * (2 * p + 2) + (ND * 4 * 2 * (p // 2) if ND % 2 else 0)
-    else:
-        u_phase = 2 * ND * ND * p * 4
-    dirs = 4 * ND if p >= 3 else 4 * ND * ND
-    return (2 * NP * ND * 4 + u_phase + 38 * ND * ND + dirs + x_phase + (4 * (NP - ND) + 2 * ND) * ND * 4
-            + (2 * ND * ne + 2 * ne) * 4 + 2 * (1 + ne) * NP * 4 + 5 * NP * 4 + (2 * NP + 1 + ne * (2 * p + 2 * NP)) * 4)
-
-
-def flops_element_direct_per_elem(p: int, ne: int, nq: int) -> float:
-    """The same for the direct form on a rule of nq points (the symmetric
-    rules): U = Phi c 2 nq N_p 4, per point 38 (the flux without H_alpha),
-    V = Dr G_r + Ds G_s 4 nq N_p 4, the lift, update and traces as above."""
-    NP = (p + 1) * (p + 2) // 2
-    ND = p + 1
-    return (2 * nq * NP * 4 + 38 * nq + 4 * nq * NP * 4
-            + (2 * ND * ne + 2 * ne) * 4 + 2 * (1 + ne) * NP * 4 + 5 * NP * 4 + (2 * NP + 1 + ne * (2 * p + 2 * NP)) * 4)
+    inst, flops = nq * 20.0, nq * 29.0
+    if p <= 3:
+        inst, flops = inst + nq * 3.0, flops + nq * 6.0
+    inst, flops = inst + 4 * NP * 7.0 / 3.0, flops + 4 * NP * 4.0
+    if p == 1:
+        inst, flops = inst + 4 * ne * 9.0, flops + 4 * ne * 15.0
+    return flops, inst
 
 
 def bytes_element_tc_per_elem(p: int, ne: int) -> float:
@@ -150,27 +111,15 @@ def _src_hash(*names) -> str:
     return h.hexdigest()[:16]
 
 
-# DRAM bytes per launch of the element kernel (dram__bytes_read.sum +
+# DRAM bytes per launch of the float64 element kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum) from one ncu capture, keyed by the hash of the code of
-# the kernel's source files (dg_element.cu and the device headers, comments
-# aside) it was taken on, and the volume rule when it is not the collapsed grid;
-# a code change voids the entry.
+# the kernel's source files (dg_split.cuh and the device headers, comments aside) it
+# was taken on, and the volume rule when it is not the collapsed grid; a code change
+# voids the entry.
 TRAFFIC = {
-    # k_element_sf<3,4,0>, stage-2 launch (reads u^n), 256x256 p=3 vortex (one ncu capture)
-    "d9a87cb5b2bffedf": 119098624 + 43275520,
-}
-
-
-# Float64 thread instructions per element of one element-kernel launch
-# (DFMA + DMUL + DADD: sm__sass_thread_inst_executed_op_d{fma,mul,add}_pred_on.sum
-# over the elements) from one ncu capture, keyed like TRAFFIC.  The float64 pipe
-# takes an FMA, a multiply or an add in the same issue slot, so these against
-# the pipe's FMA rate (half the flop peak) tell how full the kernel keeps the
-# pipe, whatever its mix of FMAs and single operations.
-FP64_INST = {
-    # k_element_sf<3,4,0>, stage-2 launch, 256x256 p=3 vortex: 1,512 DFMA + 289.2 DMUL
-    # + 240.6 DADD per element (the stage-1 launch, without u^n, has 40 fewer)
-    "d9a87cb5b2bffedf": 1512.0 + 289.1875 + 240.59375,
+    # k_element_split<3,4,0>, stage-2 launch (reads u^n), 256x256 p=3 vortex; then <3,4,12>
+    "ad67caf4880f07db": 119143936 + 44009984,
+    "ad67caf4880f07db:symmetric": 119143680 + 43739648,
 }
 
 
@@ -702,8 +651,7 @@ def run_rules(n: int = 256, steps: int = 100):
                         "dof_updates_per_s": _dof_per_step(m.N, p) * steps / (ms * 1e-3),
                         "element_ms_per_launch": el_ms / max(1, el_n)}
                 if prec == "fp64":
-                    fl = (flops_element_direct_per_elem(p, m.ne, m.nq) if rule == "symmetric"
-                          else flops_element_per_elem(p, m.ne)) * m.N
+                    fl = fp64_split_per_elem(p, m.ne, m.nq)[0] * m.N
                     line["element_fp64_tflops"] = fl / (line["element_ms_per_launch"] * 1e-3) / 1e12
                 print(json.dumps(line), flush=True)
             del m
@@ -966,26 +914,21 @@ def run_ours(args, world, rank, local):
         el_n, el_ms = ktimes.get("element", (0, 0.0))
         avg_el_ms = el_ms / max(1, el_n)
         if prec == "fp64":
-            if args.vol_rule == "symmetric":
-                flops = flops_element_direct_per_elem(p, ne, m.nq) * m.N
-            else:
-                flops = flops_element_per_elem(p, ne) * m.N
+            flops_e, inst_e = fp64_split_per_elem(p, ne, m.nq)
+            flops = flops_e * m.N
             achieved = flops / (avg_el_ms * 1e-3) / 1e12
-            khash = _src_hash("dg_element.cu", "dg_device.cuh", "dg_tcgen05.cuh")
+            khash = _src_hash("dg_split.cuh", "dg_device.cuh", "dg_edgeint.cuh", "dg_tcgen05.cuh")
             if args.vol_rule != "collapsed":
                 khash += ":" + args.vol_rule
-            roofline = {"bound": "alu", "kernel": "k_element_sf (float64 FMA pipe)",
+            ach_i = inst_e * m.N / (avg_el_ms * 1e-3) / 1e12
+            roofline = {"bound": "alu", "kernel": "k_element_split (float64 pipe; contractions on tcgen05)",
                         "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                         "frac": achieved / fp64_peak if fp64_peak else None, "traffic": TRAFFIC.get(khash),
                         "peak_source": "measured live: dg_probe_fma_rate float64 FMA chain",
-                        "flops_per_launch": flops, "avg_launch_ms": avg_el_ms}
-            ipe = FP64_INST.get(khash)
-            if ipe is not None and fp64_peak:
-                ach_i = ipe * m.N / (avg_el_ms * 1e-3) / 1e12
-                roofline["fp64_issue"] = {"inst_per_elem": ipe, "achieved": ach_i, "peak": fp64_peak / 2,
-                                          "unit": "T float64 instructions/s", "frac": ach_i / (fp64_peak / 2)}
-            else:
-                roofline["fp64_issue"] = None
+                        "flops_per_launch": flops, "avg_launch_ms": avg_el_ms,
+                        "fp64_issue": {"inst_per_elem": inst_e, "achieved": ach_i, "peak": fp64_peak / 2,
+                                       "unit": "T float64 instructions/s", "frac": ach_i / (fp64_peak / 2)}
+                        if fp64_peak else None}
         else:
             nbytes = bytes_element_tc_per_elem(p, ne) * m.N
             achieved = nbytes / (avg_el_ms * 1e-3) / 1e9
