@@ -16,7 +16,7 @@
  *
  * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 20 us
  * (p = 1), 66 -> 29 (p = 2), 87 -> 37 (p = 3), 105 -> 45 (p = 4), 124 -> 54 (p = 5);
- * k_face_mixed 88 -> 48 us (p = 3), 403 -> 185 us (512 x 512, p = 4).  Against 113-bit arithmetic the
+ * k_face_mixed 88 -> 42 us (p = 3), 403 -> 173 us (512 x 512, p = 4).  Against 113-bit arithmetic the
  * error is 0.75-1.0 of the float64 form's (rms) over still, slow, supersonic and
  * discontinuous states.
  *
@@ -135,13 +135,15 @@ DG_HD long long shr_rn(long long x, int d) {
 }
 
 // x 2^(1083 - e), truncated toward zero, for a float64 x of biased exponent at most
-// e (e >= 63, so that a zero comes out as 0): below 2^61
+// e (e >= 63, so that a zero comes out as 0): below 2^61.  F32: x is a float32 number
+// (its low 29 bits are zero), here and below: the same results.
+template <bool F32 = false>
 DG_HD long long fixed_of(double x, int e, unsigned long long *magnitude = nullptr) {
   const long long b = bits_of(x);
   const int hi = (int)(b >> 32);
   const int own = (hi >> 20) & 0x7FF;
   const uint32_t mh = ((uint32_t)hi & 0xFFFFFu) | 0x100000u, l = (uint32_t)b;
-  const unsigned long long m = ((unsigned long long)((mh << 8) | (l >> 24)) << 32) | (l << 8);
+  const unsigned long long m = ((unsigned long long)((mh << 8) | (l >> 24)) << 32) | (F32 ? 0u : l << 8);
   const int d = e - own;
   const long long v = (long long)(m >> (d < 63 ? d : 63));
   if (magnitude) *magnitude = (unsigned long long)v;
@@ -165,11 +167,12 @@ DG_HD double to_double(long long F, int X) {
 // 1/m for the mantissa m in [1, 2) of a float64, times 2^62: in [2^61, 2^62].
 // A float32 estimate y0 (23 bits) and its residual d = 1 - m y0, exact in 84 bits,
 // give y0 (1 + d + d^2); the next term is below 2^-64.
+template <bool F32 = false>
 DG_HD long long recip_mantissa(double x) {
   const long long b = bits_of(x);
   const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
   const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
-  const int ah = (int)((mh << 10) | (lo >> 22)), al = (int)((lo << 9) & 0x7FFFFFFFu);   // m 2^61 = ah 2^31 + al
+  const int ah = (int)((mh << 10) | (lo >> 22)), al = F32 ? 0 : (int)((lo << 9) & 0x7FFFFFFFu);   // m 2^61 = ah 2^31 + al
   const float f = float_of_bits(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
   const int y = to_int(rcp32(f) * 8388608.0f);                                          // [2^22, 2^23]
   // e = 2^84 - y m 2^61 = d 2^84
@@ -247,6 +250,7 @@ DG_HD FaceFix face_fix(double sx, double sy, double hk) {
 
 // l F_hat as lax_friedrichs_edge; g1 = gamma - 1 in fixed_of scale with its own
 // biased exponent eg.  False: this point is not in the range above, nothing written.
+template <bool F32 = false>
 DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix &g, double sx, double sy, long long g1,
                            int eg, double out[4]) {
   using namespace fx;
@@ -277,17 +281,17 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   for (int s = 0; s < 2; ++s) {
     const double *u = s ? ur : ul;
     const int re = s ? rR : rL;
-    const long long y = recip_mantissa(u[0]);                   // 1/rho = y 2^(961 - re)
+    const long long y = recip_mantissa<F32>(u[0]);                   // 1/rho = y 2^(961 - re)
     const long long yc = y < (1ll << 62) ? y : (1ll << 62) - 1;
     const long long I = yc >> (1 + re - r0);                    // 1/rho = I 2^(962 - r0)
     unsigned long long ax, ay;
-    const Half2x31 Mx = cut(fixed_of(u[1], em, &ax)), My = cut(fixed_of(u[2], em, &ay));
+    const Half2x31 Mx = cut(fixed_of<F32>(u[1], em, &ax)), My = cut(fixed_of<F32>(u[2], em, &ay));
     const long long mn = mul(Mx, Sx) + mul(My, Sy);
     const long long sn = mn >> 63;                              // X = em + es - r0 - 1080
     w[s] = ((long long)umul((unsigned long long)((mn ^ sn) - sn), (unsigned long long)I * 4) ^ sn) - sn;
     const unsigned long long q = umul(ax, ax * 4) + umul(ay, ay * 4);
     const long long K = (long long)umul(q, (unsigned long long)I * 4);   // |m|^2 / rho, X = 2 em - r0 - 1080
-    Pf[s] = (fixed_of(u[3], eE + 6) - shr(K, dK)) * 64;         // p / (gamma - 1), X = eE - 1083
+    Pf[s] = (fixed_of<F32>(u[3], eE + 6) - shr(K, dK)) * 64;         // p / (gamma - 1), X = eE - 1083
     ok &= Pf[s] > 0;
     const int z = clz64((unsigned long long)Pf[s]) - 2;         // Pf 2^z in [2^61, 2^62)
     const long long Pn = (long long)((unsigned long long)Pf[s] << (z & 63));

@@ -30,94 +30,96 @@
 namespace dg {
 namespace {
 
-// Edge flux of the mixed-precision modes, one thread per edge.  The two traces
-// are float32 (exact results of the tensor-core contraction) and are widened
-// exactly; the local Lax-Friedrichs flux is evaluated as in k_face (edge_flux_fixed) at
-// the NE edge points, with the right element's trace at the reversed point
-// (Eq. edgeint).  Written per
-// edge: l F_hat at the points rounded to float32 (the lift columns of GEMM 2), and
-// the float64 integral of l F_hat against the constant mode,
-// fmean_m = sum_k omega_k phi_1 l F_hat_{k,m} (Algorithm 2 for j = 1; the
-// Gauss-Legendre weights are symmetric, so it is the same from both sides).
+// Edge flux of the mixed-precision modes, one thread per edge point: a block takes 32
+// edges, warp k their k-th points.  The two traces are float32 (exact results of the
+// tensor-core contraction) and are widened exactly; the local Lax-Friedrichs flux is
+// evaluated as in k_face (edge_flux_fixed), with the right element's trace at the
+// reversed point (Eq. edgeint).  Written per edge: l F_hat at the points rounded to
+// float32 (the lift columns of GEMM 2), and the float64 integral of l F_hat against
+// the constant mode, fmean_m = sum_k omega_k phi_1 l F_hat_{k,m} (Algorithm 2 for
+// j = 1; the Gauss-Legendre weights are symmetric, so it is the same from both
+// sides), summed in the order of k from shared memory.
 // BND: the launch covers the boundary faces [f0, f1) = [0, Fb) (a ghost state on
 // the right, Algorithm 2); otherwise the interior faces [Fb, F), in a separate
 // instantiation so that the common case carries no boundary code.
-constexpr int kMixedFaceThreads = 64;
+// Bound by its integer instructions (ALU pipe 58 % busy) and their latency.  One point
+// a thread instead of one edge: 196,608 edges in 64-thread blocks were 1.7 rounds of
+// the GPU (p = 3: 47.9 -> 41.8 us); at 64 registers, 1,024 threads an SM instead of 768
+// (512 x 512, p = 4: 185 -> 173 us with both; p = 5 68 -> 59 us, p = 1 26.6 -> 25.0).
+constexpr int kMixedEdges = 32;                // edges of a block, one per lane
 template <int NE, bool BND>
-__global__ void __launch_bounds__(kMixedFaceThreads, 768 / kMixedFaceThreads)
+__global__ void __launch_bounds__(kMixedEdges * NE, 1024 / (kMixedEdges * NE))
 k_face_mixed(const float *__restrict__ trace, float *__restrict__ fhat, double *__restrict__ fmean,
              const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const FaceFix *__restrict__ ff,
              const double *__restrict__ Lf, const double *__restrict__ bstate, int np, int64_t N, int64_t f0,
              int64_t f1, GammaFix gf, int *err) {
-  constexpr int NF = 3 * NE;
-  bool ok = true;
-  // block b takes the b-th of gridDim.x equal slices of the edges
-  const int64_t F = f1 - f0;
-  const int64_t lo = f0 + F * blockIdx.x / gridDim.x, hi = f0 + F * (blockIdx.x + 1) / gridDim.x;
-  for (int64_t f = lo + threadIdx.x; f < hi; f += blockDim.x) {
+  constexpr int NF = 3 * NE, LD = NE * kMixedEdges + 8;        // + 8: the sums below read free of conflicts
+  __shared__ double sF[M * LD];
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const int64_t fb = f0 + (int64_t)blockIdx.x * kMixedEdges, f = fb + lane;
+  if (f < f1) {
     const FaceConn cn = conn[f];
     const FaceGeo *g = fg + f;
     const FaceFix fix = ff[f];
     const double2 s2 = *reinterpret_cast<const double2 *>(&g->sx);
     const double sx = s2.x, sy = s2.y;
     // [N][NF][M] float32: one point's four values are one aligned float4
-    constexpr bool bnd = BND;
-    const int64_t el = checked(cn.l, N, err);
-    const float4 *tl = reinterpret_cast<const float4 *>(trace) + (size_t)el * NF + checked(cn.L, 3, err) * NE;
-    const float4 *tr = reinterpret_cast<const float4 *>(trace) + (size_t)(bnd ? el : checked(cn.r, N, err)) * NF +
-                       (bnd ? 0 : checked(cn.R, 3, err) * NE);
-    float4 *dst = reinterpret_cast<float4 *>(fhat) + (size_t)f * NE;
-    double sm[M] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 1
-    for (int k = 0; k < NE; ++k) {
-      const float4 a = tl[k];
-      double Fh[M], ur[M];
-      const double ul[M] = {tc::f32_to_f64(a.x), tc::f32_to_f64(a.y), tc::f32_to_f64(a.z), tc::f32_to_f64(a.w)};
-      if (bnd) {
-        ghost_state(cn.r, ul, g->nx, g->ny, bstate + ((size_t)f * NE + k) * M, ur);
-      } else {
-        const float4 b = tr[NE - 1 - k];
-        ur[0] = tc::f32_to_f64(b.x);
-        ur[1] = tc::f32_to_f64(b.y);
-        ur[2] = tc::f32_to_f64(b.z);
-        ur[3] = tc::f32_to_f64(b.w);
-      }
-      // The results are rounded to float32 below.  On faces along the axes of a
-      // uniform mesh, between equal traces, they are products of a float32 and a
-      // number of a few bits, and lie in the middle between two float32 values as
-      // often as not: the last float64 bit decides.  Such points take the float64
-      // form, so that the stored flux does not depend on the form of the others.
-      bool done = edge_flux_fixed(ul, ur, fix, sx, sy, gf.g1, gf.eg, Fh);
-      if (done) {
-        bool tie = false;
-#pragma unroll
-        for (int m = 0; m < M; ++m) tie |= near_f32_tie(Fh[m]);
-        done = !tie;
-      }
-      if (!done) {
-        double o[M];
-        if (bnd) {
-          double x[M], y[M];
-#pragma unroll
-          for (int m = 0; m < M; ++m) { x[m] = ul[m]; y[m] = ur[m]; }
-          ok &= lax_friedrichs_edge_call(x, y, g, gf.gamma, o);
-        } else {
-          ok &= lax_friedrichs_edge_f32_call(a, tr[NE - 1 - k], g, gf.gamma, o);
-        }
-#pragma unroll
-        for (int m = 0; m < M; ++m) Fh[m] = o[m];
-      }
-      const double w = Lf[k * np];           // omega_k phi_1, the same on the three faces
-#pragma unroll
-      for (int m = 0; m < M; ++m) sm[m] = fma(w, Fh[m], sm[m]);
-      dst[k] = make_float4(tc::f64_to_f32(Fh[0]), tc::f64_to_f32(Fh[1]), tc::f64_to_f32(Fh[2]),
-                           tc::f64_to_f32(Fh[3]));
+    const float4 *t4 = reinterpret_cast<const float4 *>(trace);
+    const float4 a = t4[(size_t)checked(cn.l, N, err) * NF + checked(cn.L, 3, err) * NE + k];
+    float4 b;
+    double Fh[M], ur[M];
+    const double ul[M] = {tc::f32_to_f64(a.x), tc::f32_to_f64(a.y), tc::f32_to_f64(a.z), tc::f32_to_f64(a.w)};
+    if constexpr (BND) {
+      ghost_state(cn.r, ul, g->nx, g->ny, bstate + ((size_t)f * NE + k) * M, ur);
+    } else {
+      b = t4[(size_t)checked(cn.r, N, err) * NF + checked(cn.R, 3, err) * NE + (NE - 1 - k)];
+      ur[0] = tc::f32_to_f64(b.x);
+      ur[1] = tc::f32_to_f64(b.y);
+      ur[2] = tc::f32_to_f64(b.z);
+      ur[3] = tc::f32_to_f64(b.w);
     }
-    double2 *dm = reinterpret_cast<double2 *>(fmean + (size_t)f * M);
-    dm[0] = make_double2(sm[0], sm[1]);
-    dm[1] = make_double2(sm[2], sm[3]);
+    // The results are rounded to float32 below.  On faces along the axes of a
+    // uniform mesh, between equal traces, they are products of a float32 and a
+    // number of a few bits, and lie in the middle between two float32 values as
+    // often as not: the last float64 bit decides.  Such points take the float64
+    // form, so that the stored flux does not depend on the form of the others.
+    bool done = edge_flux_fixed<!BND>(ul, ur, fix, sx, sy, gf.g1, gf.eg, Fh);
+    if (done) {
+      bool tie = false;
+#pragma unroll
+      for (int m = 0; m < M; ++m) tie |= near_f32_tie(Fh[m]);
+      done = !tie;
+    }
+    if (!done) {
+      double o[M];
+      bool ok;
+      if constexpr (BND) {
+        double x[M], y[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) { x[m] = ul[m]; y[m] = ur[m]; }
+        ok = lax_friedrichs_edge_call(x, y, g, gf.gamma, o);
+      } else {
+        ok = lax_friedrichs_edge_f32_call(a, b, g, gf.gamma, o);
+      }
+      if (!ok) atomicOr(err, kErrNonPhysical);
+#pragma unroll
+      for (int m = 0; m < M; ++m) Fh[m] = o[m];
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) sF[m * LD + k * kMixedEdges + lane] = Fh[m];
+    reinterpret_cast<float4 *>(fhat)[(size_t)f * NE + k] =
+        make_float4(tc::f64_to_f32(Fh[0]), tc::f64_to_f32(Fh[1]), tc::f64_to_f32(Fh[2]), tc::f64_to_f32(Fh[3]));
   }
-  if (!ok) atomicOr(err, kErrNonPhysical);
+  __syncthreads();
+  for (int i = threadIdx.x; i < kMixedEdges * M; i += kMixedEdges * NE) {
+    const int e = i / M, m = i % M;
+    if (fb + e >= f1) break;
+    double sm = 0.0;
+#pragma unroll
+    for (int q = 0; q < NE; ++q)               // omega_k phi_1, the same on the three faces
+      sm = fma(Lf[q * np], sF[m * LD + q * kMixedEdges + e], sm);
+    fmean[(size_t)fb * M + i] = sm;
+  }
 }
 
 // Self-check of the integer float64 <-> float32 conversions against the hardware
@@ -189,17 +191,17 @@ MixedBuffers mixed_buffers(const dg_mesh *m, double *trace, double *fhat) {
 
 int launch_face_flux_mixed(const dg_mesh *m, const MixedBuffers &b, void *stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  // an edge a thread, not a resident grid (k_face)
-  auto grid = [](int64_t n) { return (unsigned)((n + kMixedFaceThreads - 1) / kMixedFaceThreads); };
+  // an edge point a thread, not a resident grid (k_face)
+  auto grid = [](int64_t n) { return (unsigned)((n + kMixedEdges - 1) / kMixedEdges); };
   const int64_t inner = m->F - m->Fb;
 #define FACE(NE)                                                                                          \
   do {                                                                                                    \
     if (inner > 0)                                                                                        \
-      k_face_mixed<NE, false><<<grid(inner), kMixedFaceThreads, 0, s>>>(                                  \
+      k_face_mixed<NE, false><<<grid(inner), kMixedEdges * NE, 0, s>>>(                                   \
           b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N, \
           m->Fb, m->F, gamma_fix(m->gamma), m->err_flag);                                                 \
     if (m->Fb > 0)                                                                                        \
-      k_face_mixed<NE, true><<<grid(m->Fb), kMixedFaceThreads, 0, s>>>(                                   \
+      k_face_mixed<NE, true><<<grid(m->Fb), kMixedEdges * NE, 0, s>>>(                                    \
           b.trace, b.fhat, b.fmean, m->face_conn, m->face_geo, m->face_fix, m->tab.Lf, m->bstate, m->np, m->N, \
           0, m->Fb, gamma_fix(m->gamma), m->err_flag);                                                    \
   } while (0)
