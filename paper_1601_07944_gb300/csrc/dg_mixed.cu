@@ -42,7 +42,7 @@ namespace {
 // BND: the launch covers the boundary faces [f0, f1) = [0, Fb) (a ghost state on
 // the right, Algorithm 2); otherwise the interior faces [Fb, F), in a separate
 // instantiation so that the common case carries no boundary code.
-// Bound by its integer instructions (ALU pipe 58 % busy) and their latency.  One point
+// Bound by its integer instructions (ALU pipe 69 % busy) and their latency.  One point
 // a thread instead of one edge: 196,608 edges in 64-thread blocks were 1.7 rounds of
 // the GPU (p = 3: 47.9 -> 41.8 us); at 64 registers, 1,024 threads an SM instead of 768
 // (512 x 512, p = 4: 185 -> 173 us with both; p = 5 68 -> 59 us, p = 1 26.6 -> 25.0).

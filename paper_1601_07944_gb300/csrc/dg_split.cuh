@@ -20,8 +20,9 @@
  * float32: exact below 2^24.  (Levels 0 and 1 cannot reach that for any input;
  * from level 2 on the bound on the largest contraction, 90 terms at p = 5, is
  * above it, and a random-signed sum stays below by a factor of 10 standard
- * deviations.  Levels 4 and 5 need not be exact.)  Levels above 5 are dropped.
- * The result is the exact product to about 2^-58 of (largest input) x (largest
+ * deviations; digits built to line up with a table's would round level 2 to even,
+ * 2^-38 of the largest product.  Levels 4 and 5 need not be exact.)  Levels above
+ * 5 are dropped.  The result is the exact product to about 2^-58 of (largest input) x (largest
  * table entry), rounded once to float64: closer than the float64 sums it
  * replaces, whose every partial sum is rounded to 2^-53.
  *
