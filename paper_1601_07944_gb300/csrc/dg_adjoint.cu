@@ -156,9 +156,10 @@ k_adj_element(const double *__restrict__ u, const double *__restrict__ lam, doub
 // One (edge, point) a thread.  The float64 pipe bounds it: the transposed flux is 86
 // operations (lax_friedrichs_vjp; 141 with separate Jacobians per side and Newton
 // roots), and the narrow pipe takes two lanes a clock (131,072 elements, p = 2: 160
-// -> 110 us).
+// -> 110 us; 106 in blocks of 128, seven an SM, instead of three of 256).
+constexpr int kAdjFaceThreads = 128;
 template <int NE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kAdjFaceThreads, 7)
 k_adj_face(const double *__restrict__ T, const double *__restrict__ G, double *__restrict__ TB,
            const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg, const double *__restrict__ bstate,
            int64_t N, int64_t F, double gamma, int *err) {
@@ -644,9 +645,8 @@ k_adj_combine_sf(const double *__restrict__ uvol, const double *__restrict__ TB,
 template <int NE>
 int run_adj_face(const dg_mesh *m, const double *T, const double *G, double *TB, cudaStream_t st) {
   const int64_t nf = m->F * NE;
-  k_adj_face<NE><<<(int)((nf + kThreads - 1) / kThreads), kThreads, 0, st>>>(T, G, TB, m->face_conn, m->face_geo,
-                                                                             m->bstate, m->N, m->F, m->gamma,
-                                                                             m->err_flag);
+  k_adj_face<NE><<<(int)((nf + kAdjFaceThreads - 1) / kAdjFaceThreads), kAdjFaceThreads, 0, st>>>(
+      T, G, TB, m->face_conn, m->face_geo, m->bstate, m->N, m->F, m->gamma, m->err_flag);
   return (int)cudaGetLastError();
 }
 
