@@ -267,23 +267,24 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   const int em = (int)((mm > (200u << 20) ? mm : (200u << 20)) >> 20);
   const int r0 = rL < rR ? rL : rR, r1 = rL < rR ? rR : rL;
   const int e0 = eL < eR ? eL : eR, eE = eL < eR ? eR : eL;
-  // shift of the kinetic energy K to the scale of E, which keeps six bits free
-  // above it: K of a physical state is below E, but its container may be larger
+  // shift of the kinetic energy K to the scale of E, which is taken six bits down for
+  // the subtraction: K of a physical state is below E, but that of another may be up
+  // to 2^6 times as large
   const int dK = eE + 6 - 2 * em + r0 - 2;
   bool ok = (r0 > 723) & (r1 < 1323) & (r1 - r0 <= 4) & (e0 > 723) & (eE < 1323) & (eE - e0 <= 4) & (em < 1323) &
             (dK >= 0) & (g.es > 0);
   if (!ok) return false;
   const Half2x31 Sx = cut(g.sx), Sy = cut(g.sy);
   const Half2x31 G1 = cut(g1);
-  long long w[2], Pf[2], c[2];
+  long long w[2], Pf[2], yc[2], c[2];
   int xc[2];
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const double *u = s ? ur : ul;
     const int re = s ? rR : rL;
     const long long y = recip_mantissa<F32>(u[0]);                   // 1/rho = y 2^(961 - re)
-    const long long yc = y < (1ll << 62) ? y : (1ll << 62) - 1;
-    const long long I = yc >> (1 + re - r0);                    // 1/rho = I 2^(962 - r0)
+    yc[s] = y < (1ll << 62) ? y : (1ll << 62) - 1;
+    const long long I = yc[s] >> (1 + re - r0);                 // 1/rho = I 2^(962 - r0)
     unsigned long long ax, ay;
     const Half2x31 Mx = cut(fixed_of<F32>(u[1], em, &ax)), My = cut(fixed_of<F32>(u[2], em, &ay));
     const long long mn = mul(Mx, Sx) + mul(My, Sy);
@@ -291,19 +292,25 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
     w[s] = ((long long)umul((unsigned long long)((mn ^ sn) - sn), (unsigned long long)I * 4) ^ sn) - sn;
     const unsigned long long q = umul(ax, ax * 4) + umul(ay, ay * 4);
     const long long K = (long long)umul(q, (unsigned long long)I * 4);   // |m|^2 / rho, X = 2 em - r0 - 1080
-    Pf[s] = (fixed_of<F32>(u[3], eE + 6) - shr(K, dK)) * 64;         // p / (gamma - 1), X = eE - 1083
-    ok &= Pf[s] > 0;
+    // E - K lies in (-2^60, 2^55): its sign is taken before the scaling by 2^6, which
+    // only a positive one leaves room for
+    const long long d = fixed_of<F32>(u[3], eE + 6) - shr(K, dK);
+    ok &= d > 0;
+    Pf[s] = (long long)((unsigned long long)d << 6);            // p / (gamma - 1), X = eE - 1083
+  }
+  if (!ok) return false;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
     const int z = clz64((unsigned long long)Pf[s]) - 2;         // Pf 2^z in [2^61, 2^62)
-    const long long Pn = (long long)((unsigned long long)Pf[s] << (z & 63));
+    const unsigned long long Pn = (unsigned long long)Pf[s] << z;
     // c^2 = hk P / rho, h^2 folded in: X = eE - 1083 - z - re + ek + 1
-    long long c2 = (long long)umul(umul((unsigned long long)Pn, (unsigned long long)yc * 4), (unsigned long long)g.hk * 4);
-    int x2 = eE - 1082 - z - re + g.ek;
+    long long c2 = (long long)umul(umul(Pn, (unsigned long long)yc[s] * 4), (unsigned long long)g.hk * 4);
+    int x2 = eE - 1082 - z - (s ? rR : rL) + g.ek;
     c2 = (x2 & 1) ? c2 >> 1 : c2;
     x2 += x2 & 1;
     c[s] = sqrt_fixed(c2);
     xc[s] = x2 / 2 - 30;
   }
-  if (!ok) return false;
   const int xw = em + g.es - r0 - 1080;
   int xa = xw > xc[0] ? xw : xc[0];
   xa = (xa > xc[1] ? xa : xc[1]) + 1;

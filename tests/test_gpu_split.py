@@ -242,3 +242,25 @@ def test_adjoint_boundary_and_stages(dgmod, oracle_mod):
     u1, u2 = torch.empty_like(d), torch.empty_like(d)
     m.rk_step_stages(d, dt, u1, u2)
     assert np.array_equal(got, _host(m.adjoint_step_stages(_dev(c), u1, u2, dt, _dev(lam))))
+
+
+@pytest.mark.parametrize("n", [8, 61])
+@pytest.mark.parametrize("precision", ["fp64", "tf32x3"])
+def test_non_physical_boundary_state(dgmod, precision, n):
+    """A prescribed state without pressure meets only the edge flux, which reports it
+    whatever the ratio of its kinetic energy to its energy."""
+    mesh = I.box_mesh(n, I.BC_STATE, I.BC_STATE)
+    m = dgmod.Mesh.from_mesh(mesh, 2)
+    c = m.project_function(lambda x, y: I.primitive_to_conserved(1 + 0 * x, 0.1 + 0 * x, 0.2 + 0 * x, 1 + 0 * x))
+    u = np.zeros((m.n_boundary, m.ne, 4))
+    u[..., 0] = u[..., 3] = 1.0
+    for mom in (1.3, 1.5, 2.0, 4.5, 5.0, 5.5, 5.8, 7.5, 7.9, 8.5, 20.0):
+        u[..., 1], u[..., 2] = 0.6 * mom, 0.8 * mom
+        m.set_boundary_state(_dev(u))
+        m.rhs(c, precision=precision)
+        if mom < 2.0 ** 0.5:
+            m.device_status()
+            continue
+        with pytest.raises(dgmod.DGError) as err:
+            m.device_status()
+        assert dgmod.STATUS[err.value.status] == "DG_ENONPHYS"
