@@ -403,9 +403,9 @@ dg_status dg_device_status(dg_mesh *mesh, void *stream);
  *   mismatches[1]: integer float32 -> float64 conversions that differ,
  *   mismatches[2]: reciprocals (three-FMA, Newton-refined and fixed-point) more
  *                  than 1 ulp from 1/x,
- *   mismatches[3]: Newton-refined square roots more than 1 ulp from sqrt(x), or
- *                  fixed-point reciprocal square roots more than 2 ulp from
- *                  1/sqrt(x) (the sound speeds of the edge flux and its adjoint).
+ *   mismatches[3]: Newton-refined and fixed-point square roots more than 1 ulp from
+ *                  sqrt(x), or fixed-point reciprocal square roots more than 2 ulp
+ *                  from 1/sqrt(x) (the sound speeds of the edge flux and its adjoint).
  * HOST int64_t[4].  Synchronous; allocates 32 bytes. */
 dg_status dg_self_test(int64_t mismatches[4], void *stream);
 

@@ -222,17 +222,17 @@ DG_HD double rsqrt_fixed(double x) {
   return of_bits((unsigned)(be - 1) >= 2046u ? 0x7FF8000000000000ll : out);
 }
 
-// sqrt(v) 2^30 for v in [2^58, 2^62): in [2^59, 2^61)
+// sqrt(v) 2^30 for v in [2^58, 2^62): in [2^59, 2^61), to 2^-55
 DG_HD long long sqrt_fixed(long long v) {
   const float f = (float)(int)(v >> 31);                        // v 2^-31, 24 bits
   const float r = rsqrt32(f);                                   // 2^15.5 / sqrt(v)
-  // b: sqrt(v) to about 2^-21 (sqrt(v) = 2^15.5 f r)
-  const int b = to_int(f * r * 181.01933598375618f) << 8;       // 2^15.5 / 2^8 = 2^7.5
-  const long long e = v - (long long)b * b;                     // |e| < 2^43
+  // b: sqrt(v) to within 2^10 (sqrt(v) = 2^15.5 f r), 2^31 at most
+  const uint32_t b = (uint32_t)to_int(f * r * 181.01933598375618f) << 8;    // 2^15.5 / 2^8 = 2^7.5
+  const long long e = v - (long long)((unsigned long long)b * b);           // |e| < 2^42
   // sqrt(v) = b + e / (2 b): the correction, 2^30 times, with a float32 quotient
   const float h = r * 2.1579186437577746e-05f * 0.5f;           // 1 / (2 sqrt(v)): 2^-15.5 / 2
-  const int t = to_int((float)(int)(e >> 11) * (h * 8589934592.0f));        // e / (2 b) 2^22
-  const long long c1 = ((long long)b << 30) + (long long)t * 256;
+  const int t = to_int((float)(int)(e >> 11) * (h * 2147483648.0f));        // e / (2 b) 2^20, below 2^31
+  const long long c1 = (long long)((unsigned long long)b << 30) + (long long)t * 1024;
   // the rest, from c1^2 / 2^62 against v / 4
   const int e1 = (int)((v >> 2) - (long long)umul((unsigned long long)c1, (unsigned long long)c1 * 4));
   const int t1 = to_int((float)e1 * (h * 4294967296.0f));

@@ -136,7 +136,33 @@ static int accuracy() {
   return !(worst < 1.0) || taken < 9 * n / 10;
 }
 
+// the square root over its whole range, denser towards both ends, and a flux whose
+// sound speeds lie at the upper end: gas at rest with rho = 1, P just below 2 and a
+// face with hk just below 1/4
+static int root() {
+  double worst = 0;
+  for (int i = 0; i < 2000000; ++i) {
+    const long long span = (1ll << 62) - (1ll << 58), r = (long long)(rng() % (unsigned long long)span) >> (i % 61);
+    const long long v = i & 1 ? (1ll << 62) - 1 - r : (1ll << 58) + r;
+    const Q e = std::fabs((Q)fx::sqrt_fixed(v) / (std::sqrt((Q)v) * 0x1p30L) - 1) / 0x1p-55L;
+    if (!(e <= worst)) worst = (double)e;
+  }
+  double flux_worst = 0;
+  for (int i = 0; i < 30; ++i) {
+    const double u[4] = {1.0, 0.0, 0.0, 2.0 - std::ldexp(1.0, i - 50)};
+    const double h = std::sqrt(0.25 * (1.0 - std::ldexp(1.0, i - 50)) / (1.4 * 0.4));
+    const Face a = face(h, 0.3, 1.4);
+    double o[4];
+    if (!flux(u, u, a, o)) return 1;
+    const double e = error(u, u, a, o);
+    if (!(e <= flux_worst)) flux_worst = e;
+  }
+  std::printf("root worst %g 2^-55, flux worst %g\n", worst, flux_worst);
+  return !(worst < 1.0) || !(flux_worst < 1.0);
+}
+
 int main(int argc, char **argv) {
+  if (!std::strcmp(argv[1], "root")) return root();
   if (!std::strcmp(argv[1], "refuse")) return refuse();
   if (!std::strcmp(argv[1], "accuracy")) return accuracy();
   return 2;
@@ -156,7 +182,7 @@ def driver(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("what", ["refuse", "accuracy"])
+@pytest.mark.parametrize("what", ["refuse", "accuracy", "root"])
 def test_edge_flux_fixed(driver, what):
     r = subprocess.run([driver, what], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.returncode, r.stdout)
