@@ -21,8 +21,8 @@
  * discontinuous states.
  *
  * A point whose sides differ by more than 2^4 in density or energy, whose state is
- * not physical or not finite, or whose exponents are far from one (beyond 2^300)
- * is left to the float64 form: edge_flux_fixed returns false and writes nothing.
+ * not physical or not finite, whose exponents are far from one (beyond 2^300), or
+ * whose (gamma - 1) P w may be below the normal range, is left to the float64 form: edge_flux_fixed returns false and writes nothing.
  */
 #pragma once
 
@@ -271,8 +271,10 @@ DG_HD bool edge_flux_fixed(const double ul[4], const double ur[4], const FaceFix
   // the subtraction: K of a physical state is below E, but that of another may be up
   // to 2^6 times as large
   const int dK = eE + 6 - 2 * em + r0 - 2;
+  // the last: below it H's exponent, eE + (em - r0 + es - 1080) + eg - 957 less up to 63
+  // leading zeros, could be negative (P w of the smallest normal numbers and less)
   bool ok = (r0 > 723) & (r1 < 1323) & (r1 - r0 <= 4) & (e0 > 723) & (eE < 1323) & (eE - e0 <= 4) & (em < 1323) &
-            (dK >= 0) & (g.es > 0);
+            (dK >= 0) & (g.es > 0) & (eE + em - r0 + g.es + eg >= 2100);
   if (!ok) return false;
   const Half2x31 Sx = cut(g.sx), Sy = cut(g.sy);
   const Half2x31 G1 = cut(g1);

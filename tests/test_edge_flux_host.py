@@ -161,7 +161,36 @@ static int root() {
   return !(worst < 1.0) || !(flux_worst < 1.0);
 }
 
+// exponents over the whole range that the fixed point may take: whatever is taken is
+// accurate (an error far below the smallest normal number counts for nothing)
+static int range() {
+  double worst = 0;
+  long taken = 0;
+  for (int i = 0; i < 1500000; ++i) {
+    const double rho = std::ldexp(U(1, 2), (int)U(-302, 302)), e = std::ldexp(U(1, 2), (int)U(-302, 302));
+    const double f = i % 3 == 0 ? U(0, 0.9) : std::exp(U(-700, 0)), gamma = 1.0 + std::exp(U(-8, 1));
+    double s[2][4], o[4];
+    for (int k = 0; k < 2; ++k) {
+      s[k][0] = rho * U(1, 2);
+      s[k][3] = e * U(1, 2);
+      const double m = std::sqrt(s[k][0]) * std::sqrt(s[k][3]) * f * U(0.5, 1), t = U(0, 6.28);
+      s[k][1] = m * std::cos(t);
+      s[k][2] = i % 5 ? m * std::sin(t) : 0.0;
+    }
+    const Face a = face(std::ldexp(1.0, (int)U(-290, 290)), U(0, 6.28), gamma);
+    if (!flux(s[0], s[1], a, o)) continue;
+    ++taken;
+    bool tiny = true;                                       // results below 2^-960: float64's own range ends here
+    for (int k = 0; k < 4; ++k) tiny &= std::fabs(o[k]) < 0x1p-960;
+    const double x = error(s[0], s[1], a, o);
+    if (!tiny && !(x <= worst)) worst = x;
+  }
+  std::printf("taken %ld worst %g\n", taken, worst);
+  return !(worst < 1.0) || taken < 300000;
+}
+
 int main(int argc, char **argv) {
+  if (!std::strcmp(argv[1], "range")) return range();
   if (!std::strcmp(argv[1], "root")) return root();
   if (!std::strcmp(argv[1], "refuse")) return refuse();
   if (!std::strcmp(argv[1], "accuracy")) return accuracy();
@@ -182,7 +211,7 @@ def driver(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("what", ["refuse", "accuracy", "root"])
+@pytest.mark.parametrize("what", ["refuse", "accuracy", "root", "range"])
 def test_edge_flux_fixed(driver, what):
     r = subprocess.run([driver, what], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.returncode, r.stdout)
