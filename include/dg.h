@@ -206,6 +206,10 @@ dg_status dg_project_ic(dg_mesh *mesh, const double *u, double *c, void *stream)
  *   F_hat = (F(U_l).n + F(U_r).n)/2 - alpha (U_r - U_l)/2,
  *   alpha = max(|v_l.n| + c_l, |v_r.n| + c_r),
  * evaluated once per edge.  c, r: DEVICE [N][4][N_p], must not alias.
+ * Range (float64, here and in the calls that step or transpose it): values of any
+ * size up to 2^1007, as far as the fluxes' products stay finite; on large meshes one
+ * element's values of a variable that are all below 2^-959 have an error of 2^-1017
+ * instead of a relative one.
  * Asynchronous. */
 dg_status dg_rhs(dg_mesh *mesh, const double *c, double *r, dg_precision prec, void *stream);
 

@@ -151,7 +151,6 @@ struct Group {
   }
 };
 
-__device__ __forceinline__ uint32_t nan_mask(uint32_t mx) { return mx >= (1980u << 20) ? 0x7FF80000u : 0u; }
 template <int N>
 __device__ __forceinline__ uint32_t max_hi(const double *v) {
   uint32_t m = 0;
@@ -246,7 +245,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
     // ---- u: values at the points, edge traces ----
     uint32_t mx = g.pair_max(sMxA, max_hi<NPH>(v));
     int E = row_exp(mx);
-    uint32_t nan = nan_mask(mx);
+    uint32_t nan = row_nan(mx);
     store_half<A::K1H, NPH>(g, tA, A::CA, v, E);
     if (!g.operands_ready()) return false;
     issue(C1{}, CK{}, A::oU);
@@ -272,7 +271,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
     to_faces(Tr, E + ex[kTabT] + 5);
     // ---- lb: cotangents of the edge fluxes and of G_r, G_s ----
     E = row_exp(mxl);
-    nan = nan_mask(mxl);
+    nan = row_nan(mxl);
     store_half<A::K1H, NPH>(g, tA, A::CA, lb, E);
     if (!g.operands_ready()) return false;
     issue(C3{}, CK{}, A::oG);
@@ -315,7 +314,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
     // ---- transposed interpolation ----
     mx = sMxG[rm * 32 + rel];
     E = row_exp(mx);
-    nan = nan_mask(mx);
+    nan = row_nan(mx);
     double b[QH];
 #pragma unroll
     for (int i = 0; i < QH; ++i) b[i] = h * QH + i < NQ ? sU[((h * QH + i) * M + rm) * LD + rel] : 0.0;
@@ -383,7 +382,7 @@ k_adj_sum_split(const double *__restrict__ uvol, const double *__restrict__ TB, 
     }
     load(next, f);
     g.wait_mma();
-    read_half<A::N2, NPH>(g, E + ex + 5, nan_mask(mx), [&](int i, double x) {
+    read_half<A::N2, NPH>(g, E + ex + 5, row_nan(mx), [&](int i, double x) {
       if (h * NPH + i < NP && live) out[o + i] = fma(s, x, r[i < NPH ? i : 0]);
     });
     return g.results_read();

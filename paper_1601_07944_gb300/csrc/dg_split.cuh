@@ -35,8 +35,11 @@
  * which the other groups fill only in part.  The error of the right-hand side
  * against an 80-bit reference falls by 1.5 (p = 2) to 2.9 (p = 5).
  *
- * A row whose largest value is not finite, or is 2^957 or more, gives NaN; values
- * below 2^-959 count as zero.
+ * A row whose largest value is below 2^-959 is taken relative to that number: its
+ * results then have an error of 2^-1017 of the largest table entry, near the end of the
+ * normal range, instead of one relative to themselves.  A row whose largest value is
+ * not finite, or is 2^1007 or more, gives NaN (a sum of 90 products with table entries
+ * below 2^8 then stays below the largest float64).
  *
  * Layout.  A tile is 32 elements = 128 rows (row = 4 e + m) = 128 TMEM lanes.  A
  * group of 256 threads works on a tile, two threads (halves h = 0, 1) per row:
@@ -135,11 +138,11 @@ struct Sp {
 
 // ---- digits ---------------------------------------------------------------
 
-// biased exponent that values are taken relative to: rows below 2^-959 count as zero
-__device__ __forceinline__ int row_exp(uint32_t hi_max) {
-  const int e = (int)(hi_max >> 20);
-  return e < 64 ? 4000 : e;
-}
+// biased exponent that a row's values are taken relative to: 64 at least, so that the
+// digits of a zero (exponent 0, its leading bit taken as set) are shifted out
+__device__ __forceinline__ int row_exp(uint32_t hi_max) { return max((int)(hi_max >> 20), 64); }
+// ones in the exponent for a row out of range (from_levels)
+__device__ __forceinline__ uint32_t row_nan(uint32_t hi_max) { return hi_max >= (2030u << 20) ? 0x7FF80000u : 0u; }
 
 // x 2^(1081 - E) truncated, plus 512 in every digit: the digits + 512, ten bits each
 // (the top one eleven)
@@ -188,7 +191,8 @@ __device__ __forceinline__ void store_digits8(uint32_t tA, int ca, const double 
 }
 
 // sum_L D_L 2^(-10 L) with the row's and the table's exponents -> float64, rounded
-// once.  xb = E + table exponent + 5: the result's biased exponent is xb + 1 - clz.
+// once.  xb = E + table exponent + 5: the result's biased exponent is xb + 1 - clz, at
+// least 7 + table exponent.
 // nan: all ones in the exponent where the row was out of range.
 __device__ __forceinline__ double from_levels(const float *d, int xb, uint32_t nan) {
   // (level 5 joins level 4 in float32: the sum's rounding is below level 5's leading bits)
@@ -464,7 +468,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
     for (int i = 0; i < NPH; ++i) mx = max(mx, (uint32_t)__double2hiint(cv[i]) & 0x7FFFFFFFu);
     mx = pair_max(sMxA, mx);
     int E = row_exp(mx);
-    uint32_t nan = mx >= (1980u << 20) ? 0x7FF80000u : 0u;
+    uint32_t nan = row_nan(mx);
     if constexpr (!TRACES) {
       store_modes(cv, E);
       if (warp < 4) {
@@ -542,7 +546,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       // ---- GEMM 2's operand: half 0 [G_r | fluxes], half 1 [G_s | fluxes] ----
       mx = sMxG[rm * 32 + rel];
       E = row_exp(mx);
-      nan = mx >= (1980u << 20) ? 0x7FF80000u : 0u;
+      nan = row_nan(mx);
       const double *g = (h == 0 ? sU : sS) + rm * LD + rel;
       double uv[NPH];
 #pragma unroll
@@ -641,7 +645,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
         if (h * NPH + i < NP) mx = max(mx, (uint32_t)__double2hiint(cv[i]) & 0x7FFFFFFFu);
       mx = pair_max(sMxB, mx);
       E = row_exp(mx);
-      nan = mx >= (1980u << 20) ? 0x7FF80000u : 0u;
+      nan = row_nan(mx);
     }
     // ---- GEMM 3: edge traces of the state in cv ----
     store_modes(cv, E);

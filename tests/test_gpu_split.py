@@ -264,3 +264,37 @@ def test_non_physical_boundary_state(dgmod, precision, n):
         with pytest.raises(dgmod.DGError) as err:
             m.device_status()
         assert dgmod.STATUS[err.value.status] == "DG_ENONPHYS"
+
+
+# Rows far from one.  The Euler fluxes are homogeneous, so that gas at rest may have any
+# unit of density and energy (moving gas may not: the square of a momentum leaves the
+# range), and the adjoint is linear in its cotangent.  In units of 2^-950 the fluxes of
+# mass, jumps of 1e-10, lie below the 2^-959 that the kernel takes its smallest rows
+# relative to: an error of 2^-1017, 2^-67 of the state, 2^-49 of a residual (sums of up
+# to 90, divided by det J of 2^-5 or more).
+@pytest.mark.parametrize("k", [-950, -900, 960, 990])
+@pytest.mark.parametrize("p,ne,rule", [(1, 0, "collapsed"), (2, 0, "symmetric"), (3, 0, "collapsed"), (4, 0, "collapsed"), (5, 0, "collapsed")])
+def test_rows_far_from_one(dgmod, oracle_mod, p, ne, rule, k):
+    mesh = I.periodic_mesh(61)
+    m = dgmod.Mesh.from_mesh(mesh, p, n_edge_pts=ne, vol_rule=rule)
+    o = oracle_mod.OracleDG.from_mesh(mesh, p, n_edge_pts=ne, vol_rule=rule)
+    c = o.project_ic(_gas(0.1, 0.1, 0, 0))
+    ref, vol = o.rhs_and_volume(c)
+    scale = np.linalg.norm(vol / o.det_j()[:, None, None])
+    unit = 2.0 ** k
+    got = _host(m.rhs(_dev(c * unit))) / unit
+    assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref) + 16 * EPS * scale
+    # a step so short that the kinetic energy (which underflows) is below a rounding;
+    # in large units any motion's would overflow: a step of length zero
+    for method in ("ssp_rk3", "rk4"):
+        got = _host(m.rk_step(_dev(c * unit), 1e-9 if k < 0 else 0.0, 1, method=method)) / unit
+        if k < 0:
+            assert rel_l2(got - c, 1e-9 * ref) < 1e-4
+        else:
+            assert rel_l2(got, c) < 1e-14
+    m.device_status()
+    if p <= 3:
+        rng = np.random.default_rng(7)
+        u = o.project_ic(I.perturbed_vortex) + 0.002 * rng.standard_normal((o.N, 4, o.np))
+        lam = rng.standard_normal(u.shape)
+        assert rel_l2(_host(m.rhs_adjoint(_dev(u), _dev(lam * unit))) / unit, o.rhs_vjp(u, lam)) < 1e-12
