@@ -392,8 +392,10 @@ dg_status dg_probe_fma_rate(double *fp64_tflops, double *fp32_tflops, void *stre
 /* Failure detection (no passage of the paper): synchronises stream and reports
  * device-side failures recorded since the last call: DG_EMESH if a kernel of a library built with DG_DEBUG read a connectivity
  * index out of range (it then used index 0 instead; other builds do not check);
- * DG_ETIMEOUT if a bounded wait of the mixed-precision kernels expired (the
- * kernel then skipped its remaining work and released its resources);
+ * DG_ETIMEOUT if a bounded wait expired, of a tensor-core kernel (float64, mixed or
+ * adjoint) or of the fused stepper (the kernel then skipped its remaining work, stored
+ * no value that depends on what it waited for, and released its resources; the call's
+ * outputs are part old, part new);
  * DG_ENONPHYS if a kernel met rho <= 0 or p <= 0 (or NaN) at a volume or edge
  * quadrature point (the results of that call are then meaningless).  The record
  * is cleared.  Synchronous. */

@@ -60,6 +60,7 @@ struct Group {
   volatile int *fail;
   int *turn, *err;
   bool in_flight;
+  int waits;
 
   __device__ __forceinline__ bool sync() const {
     bar_sync(1 + sub, kSubThreads);
@@ -79,14 +80,16 @@ struct Group {
     tc::fence_after_sync();
     return ok;
   }
-  __device__ __forceinline__ void wait_mma() {
+  __device__ __forceinline__ bool wait_mma() {
     in_flight = true;
-    if (!tc::mbar_wait_sleep(mbar, phase, kSplitWaitNs, kSplitSuspendNs)) {
+    const bool done = tc::mbar_wait_sleep(mbar, phase, kSplitWaitNs, kSplitSuspendNs) && !expire_wait(err, waits++);
+    if (!done) {
       fail[sub] = 1;
       atomicOr(err, kErrTimeout);
     }
     phase ^= 1u;
     tc::fence_after_sync();
+    return done;
   }
   __device__ __forceinline__ uint32_t pair_max(uint32_t *s, uint32_t v) const {
     s[h * 128 + row] = v;
@@ -115,6 +118,7 @@ struct Group {
     mbar = tc::smem_u32(bars + sub);
     phase = 0;
     in_flight = false;
+    waits = 0;
     if (threadIdx.x < 32) tc::tmem_alloc(tc::smem_u32(slot), 512);
     if (threadIdx.x == 0) {
       for (int i = 0; i <= subs; ++i) tc::mbar_init(tc::smem_u32(bars + i), 1);
@@ -228,7 +232,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
 
   auto tile_body = [&](int tile) -> bool {
     const int e0 = tile * EB, ecount = min(EB, N - e0);
-    const bool live = rel < ecount;
+    bool live = rel < ecount;                                // (and no wait has expired: nothing is stored after one)
     const size_t orow = ((size_t)(e0 + rel) * M + rm) * NP + h * NPH;
     double v[NPH], lb[NPH];
     const double inv = live ? geo[(size_t)(e0 + rel) * GEO + 4] : 0.0;
@@ -267,7 +271,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
 #pragma unroll
     for (int i = 0; i < NPH; ++i) lb[i] *= inv;
     const uint32_t mxl = g.pair_max(sMxB, max_hi<NPH>(lb));
-    g.wait_mma();
+    live = g.wait_mma() && live;
     to_faces(Tr, E + ex[kTabT] + 5);
     // ---- lb: cotangents of the edge fluxes and of G_r, G_s ----
     E = row_exp(mxl);
@@ -275,7 +279,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
     store_half<A::K1H, NPH>(g, tA, A::CA, lb, E);
     if (!g.operands_ready()) return false;
     issue(C3{}, CK{}, A::oG);
-    g.wait_mma();
+    live = g.wait_mma() && live;
     to_faces(G, E + ex[kTabG] + 5);
     if (!g.results_read()) return false;
     issue(C1{}, CK{}, A::oR);
@@ -321,7 +325,7 @@ k_adj_split(const double *__restrict__ u, const double *__restrict__ lam, double
     store_half<A::KQ, QH>(g, tA, A::CA, b, E);
     if (!g.operands_ready()) return false;
     issue(C2{}, CV{}, A::oV);
-    g.wait_mma();
+    live = g.wait_mma() && live;
     read_half<A::N2, NPH>(g, E + ex[kTabV] + 5, nan, [&](int i, double x) {
       if (h * NPH + i < NP && live) uvol[orow + i] = x;
     });
@@ -360,7 +364,7 @@ k_adj_sum_split(const double *__restrict__ uvol, const double *__restrict__ TB, 
   double f[NFH];
   auto tile_body = [&](int tile, int next) -> bool {
     const int e = tile * EB + g.rel;
-    const bool live = e < N;
+    bool live = e < N;
     const size_t o = ((size_t)e * M + g.rm) * NP + h * NPH;
     const uint32_t mx = g.pair_max(sMx, max_hi<NFH>(f));
     const int E = row_exp(mx);
@@ -381,7 +385,7 @@ k_adj_sum_split(const double *__restrict__ uvol, const double *__restrict__ TB, 
       if (Z && on) r[i] = fma(x2, Z[o + i], r[i]);
     }
     load(next, f);
-    g.wait_mma();
+    live = g.wait_mma() && live;
     read_half<A::N2, NPH>(g, E + ex + 5, row_nan(mx), [&](int i, double x) {
       if (h * NPH + i < NP && live) out[o + i] = fma(s, x, r[i < NPH ? i : 0]);
     });

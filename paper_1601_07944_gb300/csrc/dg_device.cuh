@@ -318,6 +318,20 @@ __device__ __forceinline__ int64_t checked(int64_t i, int64_t n, int *err) {
   return i;
 }
 
+// Whether the nth completed wait of a thread is to be taken for one that expired: in
+// DG_DEBUG builds where the mesh was created with DG_DEBUG_EXPIRE = nth in the
+// environment (kept above the flag bits), so that the give-up paths can be tested
+// with every wait ending as usual.
+constexpr int kErrExpireShift = 8;
+__device__ __forceinline__ bool expire_wait(const int *err, int nth) {
+#ifdef DG_DEBUG
+  return *reinterpret_cast<const volatile int *>(err) >> kErrExpireShift == nth + 1;
+#else
+  (void)err; (void)nth;
+  return false;
+#endif
+}
+
 template <int NE>
 __device__ __forceinline__ void face_flux_points(const double *__restrict__ trace, double *__restrict__ fhat,
                                                  const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,

@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <limits>
 #include <new>
@@ -800,6 +801,10 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
     }
   }
   cudaError_t ce;
+  int err0 = 0;
+#ifdef DG_DEBUG
+  if (const char *nth = getenv("DG_DEBUG_EXPIRE")) err0 = (atoi(nth) + 1) << 8;   // expire_wait
+#endif
   if (Fb > 0 &&
       ((ce = cudaMemcpy(m->bxy, bxy.data(), sizeof(double) * Fb * ne * 2, cudaMemcpyHostToDevice)) != cudaSuccess ||
        (ce = cudaMemset(m->bstate, 0, sizeof(double) * Fb * ne * M)) != cudaSuccess)) {
@@ -814,7 +819,7 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
       (ce = cudaMemcpy(m->face_geo, fgeo.data(), sizeof(FaceGeo) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = (cudaError_t)dg::launch_face_fix(m)) != cudaSuccess ||
       (ce = cudaMemcpy(m->table_block, tb.data(), sizeof(double) * off, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (ce = cudaMemset(m->err_flag, 0, sizeof(int))) != cudaSuccess ||
+      (ce = cudaMemcpy(m->err_flag, &err0, sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (ce = (cudaError_t)dg::tc_tables(m)) != cudaSuccess ||
       (ce = (cudaError_t)dg::split_tables(m)) != cudaSuccess) {
     free_mesh(m);
@@ -1505,15 +1510,16 @@ extern "C" dg_status dg_device_status(dg_mesh *m, void *stream) {
   int flag = 0;
   DG_CUDA(cudaMemcpyAsync(&flag, m->err_flag, sizeof(int), cudaMemcpyDeviceToHost, s), "dg_device_status");
   DG_CUDA(cudaStreamSynchronize(s), "dg_device_status sync");
-  if (flag) {
+  if (flag) {                             // (a DG_DEBUG build's request for an expired wait ends here too)
     DG_CUDA(cudaMemsetAsync(m->err_flag, 0, sizeof(int), s), "dg_device_status reset");
     DG_CUDA(cudaStreamSynchronize(s), "dg_device_status sync");
     if (flag & 4)
       return fail(DG_EMESH, "a kernel read a connectivity index out of range (checked in DG_DEBUG builds)");
     if (flag & 1)
-      return fail(DG_ETIMEOUT, "a tensor-core wait in the mixed-precision kernel expired%s",
+      return fail(DG_ETIMEOUT, "a bounded wait of a tensor-core kernel or of the fused stepper expired%s",
                   (flag & 2) ? "; a non-physical state was also met" : "");
-    return fail(DG_ENONPHYS, "a non-physical state (rho <= 0 or p <= 0) was met at a quadrature point");
+    if (flag & 2)
+      return fail(DG_ENONPHYS, "a non-physical state (rho <= 0 or p <= 0) was met at a quadrature point");
   }
   return DG_OK;
 }

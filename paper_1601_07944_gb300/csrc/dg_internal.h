@@ -186,8 +186,7 @@ struct dg_mesh {
   double *host_state;          // [N][M][np] device copy used by dg_rk_step_host
   double *rk_acc;              // [N][M][np] running sum of the RK4 stages (first RK4 call)
   double *partial;             // [nblk][M] totals partials
-  int *err_flag;               // device int: bit 0 = a bounded tensor-core wait expired,
-                               //             bit 1 = a non-physical state was met
+  int *err_flag;               // device int: the bits kErrTimeout, kErrNonPhysical, kErrIndex
   double rin_min;              // smallest inscribed radius 2 area / perimeter
   double phi1;                 // the constant basis function (sqrt 2)
   int limiter;                 // dg_set_limiter: limit every stage (p = 1, float64)

@@ -375,14 +375,17 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
     tc::fence_after_sync();
     return ok;
   };
-  auto mma_wait = [&]() {
+  int waits = 0;
+  auto mma_wait = [&]() -> bool {                            // false: expired, the accumulator is not to be used
     in_flight = true;
-    if (!tc::mbar_wait_sleep(mbar, phase, kSplitWaitNs, kSplitSuspendNs)) {
+    const bool done = tc::mbar_wait_sleep(mbar, phase, kSplitWaitNs, kSplitSuspendNs) && !expire_wait(err, waits++);
+    if (!done) {
       fail[sub] = 1;
       atomicOr(err, kErrTimeout);
     }
     phase ^= 1u;
     tc::fence_after_sync();
+    return done;
   };
   // the larger of the two halves' values (a barrier of the row's two warps)
   auto pair_max = [&](uint32_t *s, uint32_t v) -> uint32_t {
@@ -440,7 +443,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
   };
   auto tile_body = [&](int tile, int next) -> bool {
     const int e0 = tile * EB, ecount = min(EB, N - e0);
-    const bool live = rel < ecount;
+    bool live = rel < ecount;                                // (and, from the last GEMM 2 on, its wait did not expire)
     const size_t orow = ((size_t)(e0 + rel) * M + rm) * NP;
     double cv[NPH], fl[NFH];
     uint32_t left = 0u;                                      // bit q: this is edge q's left element
@@ -575,7 +578,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       for (int i = 0; i < NPH; ++i) uv[i] = need_u0 && live && h * NPH + i < NP ? u0[orow + h * NPH + i] : 0.0;
       if constexpr (LATE)
         if (mode != 0) load_modes(tile, cv);
-      mma_wait();
+      live = mma_wait() && live;
       // ---- stage update ----
       {
         const int xb = E + ex[1] + 5;
@@ -654,7 +657,7 @@ k_element_split(const double *c, const double *u0, double *out, double *__restri
       gemm_digits<T::N3, T::K1>(tmem, aD, T::CA, uB + T::oB3, true);
       tc::commit(mbar);
     }
-    mma_wait();
+    live = mma_wait() && live;
     {
       const int xb = E + ex[2] + 5;
       double *dst = trace_out + (size_t)(e0 + rel) * NF * M + rm;

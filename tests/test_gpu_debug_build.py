@@ -73,3 +73,63 @@ def test_index_checking_build_runs_clean(oracle_mod):
     r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % ROOT + SCRIPT], env=env, cwd=ROOT,
                        capture_output=True, text=True, timeout=900)
     assert r.returncode == 0 and "debug build clean" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+# Waits that expire, on a mesh of the split-product kernels (61 x 61 squares).
+EXPIRE_SCRIPT = r'''
+import os, sys
+import numpy as np
+import torch
+sys.path.insert(0, ROOT)
+from paper_1601_07944_gb300 import dg, inputs as I
+lib = dg.load()
+assert lib._name.endswith("libdg_debug.so"), lib._name
+mesh = I.periodic_mesh(61)
+
+# A completed wait of every tile group is reported as expired, the nth of each thread:
+# DG_ETIMEOUT, and nothing of the kernel's last stores.  With one tile a group the
+# right-hand side's element kernel has GEMM 1's wait and one for each batch of GEMM 2,
+# the last of them before its stores; the adjoint's last kernel has one.
+def expire(nth, p, call):
+    os.environ["DG_DEBUG_EXPIRE"] = str(nth)
+    m = dg.Mesh.from_mesh(mesh, p)
+    del os.environ["DG_DEBUG_EXPIRE"]
+    c = m.project_function(I.perturbed_vortex)
+    out = torch.full_like(c, 7.0)
+    call(m, c, out)
+    try:
+        m.device_status()
+        expired = False
+    except dg.DGError as e:
+        assert dg.STATUS[e.status] == "DG_ETIMEOUT", e
+        expired = True
+    untouched = bool((out == 7.0).all())
+    call(m, c, out)                       # the request ended with the status: a call as usual
+    m.device_status()
+    return expired, untouched, out.cpu().numpy(), m
+
+for p in (1, 2, 3, 5):
+    ref = None
+    seen = []
+    for nth in range(9):
+        expired, untouched, got, m = expire(nth, p, lambda m, c, out: m.rhs(c, out=out))
+        assert untouched == expired, (p, nth, expired, untouched)
+        seen.append(expired)
+        ref = got if ref is None else ref
+        assert np.array_equal(got, ref)
+    assert seen[0] and seen[1] and not seen[-1], seen
+    if p <= 3:
+        lam = torch.randn((m.N, 4, m.np), dtype=torch.float64, device="cuda")
+        expired, untouched, _, _ = expire(0, p, lambda m, c, out: m.rhs_adjoint(c, lam, out=out))
+        assert expired and untouched
+print("debug build clean")
+'''
+
+
+def test_expired_waits_store_nothing():
+    from paper_1601_07944_gb300 import _build
+    lib = _build.build(debug=True)
+    env = dict(os.environ, DG_LIB=lib)
+    r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % ROOT + EXPIRE_SCRIPT], env=env, cwd=ROOT,
+                       capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0 and "debug build clean" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
