@@ -868,6 +868,13 @@ __device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned target, int *e
 constexpr int kSmallThreads = 128;
 constexpr int kSmallTiles[2] = {4, 8};          // elements per tile of the two variants
 
+// Blocks per SM that the stepper's registers are held to.  At p = 1 the 8-element
+// tiles take five (96 registers, no spills, instead of 122-128), which serves meshes
+// up to 6,080 elements on 152 SMs: ten SSP-RK3 steps at 5,000-6,050 elements 0.30-0.32
+// ms against 0.56 with separate launches (0.53-0.58 before the split-product kernel).
+// At p >= 2 the separate launches are the faster ones beyond four blocks.
+constexpr int small_blocks(int p, int tile) { return p == 1 && tile == 8 ? 5 : 4; }
+
 // shared memory of the stepper: the tile's phases, then the step's first state and
 // the RK4 sum [EB][M][NP], 1/det J [EB] and the elements' edges [EB][3]
 template <int P, int NE, int Q, int EBX>
@@ -878,7 +885,7 @@ struct SmallCfg {
 };
 
 template <int P, int NE, int Q, int EBX>
-__global__ void __launch_bounds__(kSmallThreads, 4)
+__global__ void __launch_bounds__(kSmallThreads, small_blocks(P, EBX))
 k_rk_small(double *c, double *S, double *A, double *trace, double *fhat, const double *__restrict__ geo,
            const int32_t *__restrict__ elem_face, const FaceConn *__restrict__ conn, const FaceGeo *__restrict__ fg,
            const FaceFix *__restrict__ ff, const double *__restrict__ bstate, const int32_t *__restrict__ elem_nbr,

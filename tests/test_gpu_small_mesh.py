@@ -101,6 +101,40 @@ def test_fused_with_limiter(dgmod, n, method):
         assert dgmod.STATUS[e.status] == "DG_ENONPHYS"   # or, without it, the run broke down
 
 
+@pytest.mark.parametrize("method", ["ssp_rk3", "rk4"])
+@pytest.mark.parametrize("p,ne,rule,n", [(1, 0, "collapsed", 41), (1, 0, "symmetric", 41), (1, 0, "collapsed", 55),
+                                         (1, 0, "symmetric", 55), (2, 0, "collapsed", 41), (2, 0, "symmetric", 41),
+                                         (3, 0, "collapsed", 41), (3, 3, "collapsed", 41), (3, 0, "symmetric", 41),
+                                         (4, 0, "collapsed", 41), (4, 0, "symmetric", 41), (5, 0, "collapsed", 41)])
+def test_fused_equals_separate_launches_8_element_tiles(dgmod, p, ne, rule, n, method):
+    """The stepper's second variant (meshes beyond 4 elements in each of 4 blocks per
+    SM), with a ragged last tile; at p = 1 up to 6,080 elements (five blocks per SM)."""
+    import torch
+    mesh = I.periodic_mesh(n)
+    m = dgmod.Mesh.from_mesh(mesh, p, n_edge_pts=ne, vol_rule=rule)
+    assert m.N > 16 * torch.cuda.get_device_properties(0).multi_processor_count and m.N % 8 == 2
+    c0 = m.project_function(I.perturbed_vortex)
+    dt = I.fixed_dt(mesh, I.perturbed_vortex, p)
+    a, kta = _run(m, c0, dt, 5, method, True)
+    b, ktb = _run(m, c0, dt, 5, method, False)
+    assert "stepper" in kta and "element" not in kta
+    assert "stepper" not in ktb and "element" in ktb
+    assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [41, 55])
+def test_fused_with_limiter_8_element_tiles(dgmod, n):
+    mesh = I.periodic_mesh(n)
+    m = dgmod.Mesh.from_mesh(mesh, 1)
+    c0 = m.limit(m.project_function(I.density_steps))
+    dt = I.fixed_dt(mesh, I.density_steps, 1)
+    m.set_limiter(True)
+    a, kta = _run(m, c0, dt, 5, "rk2", True)
+    b, ktb = _run(m, c0, dt, 5, "rk2", False)
+    assert "stepper" in kta and "element" not in kta and "stepper" not in ktb
+    assert np.array_equal(a, b)
+
+
 def test_fused_matches_oracle(dgmod, oracle_mod):
     """The fused path against the oracle's SSP-RK3 run (relative L2 <= 1e-12)."""
     mesh = I.periodic_mesh(12)
