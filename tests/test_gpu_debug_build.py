@@ -75,6 +75,21 @@ def test_index_checking_build_runs_clean(oracle_mod):
     assert r.returncode == 0 and "debug build clean" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
 
 
+def test_index_checking_build_runs_clean_on_large_meshes(oracle_mod):
+    """The same calls on 7,442 elements: the split-product kernels, their traces mode
+    and the adjoint's, a ragged last tile, for two steps."""
+    from paper_1601_07944_gb300 import _build
+    lib = _build.build(debug=True)
+    large = SCRIPT
+    for small, big in (("periodic_mesh(6)", "periodic_mesh(61)"), ("box_mesh(6,", "box_mesh(61,"), ("dt, 18", "dt, 2")):
+        assert small in large
+        large = large.replace(small, big)
+    env = dict(os.environ, DG_LIB=lib)
+    r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % ROOT + large], env=env, cwd=ROOT,
+                       capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0 and "debug build clean" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
+
+
 # Waits that expire, on a mesh of the split-product kernels (61 x 61 squares).
 EXPIRE_SCRIPT = r'''
 import os, sys
