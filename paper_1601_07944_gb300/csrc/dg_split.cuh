@@ -17,14 +17,16 @@
  * d_i e_j with i + j = L,
  *     sum_k x_k b_k = 2^s sum_L D_L 2^(-10 L),
  * and every D_L is a sum of integers of at most 2^18 that the tensor core forms in
- * float32: exact below 2^24.  (Levels 0 and 1 cannot reach that for any input;
- * from level 2 on the bound on the largest contraction, 90 terms at p = 5, is
- * above it, and a random-signed sum stays below by a factor of 10 standard
- * deviations; digits built to line up with a table's would round level 2 to even,
- * 2^-38 of the largest product.  Levels 4 and 5 need not be exact.)  Levels above
- * 5 are dropped.  The result is the exact product to about 2^-58 of (largest input) x (largest
- * table entry), rounded once to float64: closer than the float64 sums it
- * replaces, whose every partial sum is rounded to 2^-53.
+ * float32: exact below 2^24.  Levels 0 and 1 stay below that for any operand (by 5 % at
+ * p = 5; tests/test_split_digits.py bounds every table), levels 2 and 3 too except in
+ * GEMM 2: level 2 there at p = 4 and 5 (up to 1.2 and 1.7 times 2^24), level 3 from p = 3
+ * on.  To pass it an operand has to line up with a table column digit by digit: sums of
+ * random sign stay below by ten standard deviations.  (Levels 4 and 5 need not be exact.)
+ * Levels above 5 are dropped.  The result is then the exact product to about 2^-58 of
+ * (largest input) x (largest table entry), rounded once to float64: closer than the
+ * float64 sums it replaces, whose every partial sum is rounded to 2^-53.  (Such an operand
+ * would lose a unit of level 2, 2^-38 of the largest product, or of level 3, 2^-48, at
+ * each of GEMM 2's K steps.)
  *
  * Measured (256 x 256 mesh, 131,072 elements, one launch of a stage, k_element_sf
  * -> here): p = 1 0.108 -> 0.084 ms, p = 2 0.265 -> 0.127, p = 3 0.498 -> 0.181,
