@@ -1010,7 +1010,7 @@ int run_rk_small(dg_mesh *m, double *c, double dt, int nsteps, int method, cudaS
   // one tile per block (the variant was chosen so that they are all resident);
   // the edge phase spreads its points over the same blocks
   const int64_t nb = (m->N + EBX - 1) / EBX;
-  cudaError_t e = cudaMemsetAsync(m->gbar, 0, 2 * sizeof(unsigned), s);
+  cudaError_t e = cudaMemsetAsync(m->gbar, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return (int)e;
   double *S = m->stage, *A = m->rk_acc, *tr = m->trace, *fh = m->fhat;
   const double *geo = m->geo, *bst = m->bstate;

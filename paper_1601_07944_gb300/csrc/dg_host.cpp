@@ -766,7 +766,7 @@ extern "C" dg_status dg_mesh_create(const dg_mesh_desc *d, dg_mesh **out) {
   DG_ALLOC(m->partial, sizeof(double) * m->totals_blocks * M, "totals partials");
   DG_ALLOC(m->totals_dev, sizeof(double) * M, "totals");
   DG_ALLOC(m->err_flag, sizeof(int), "error flag");
-  DG_ALLOC(m->gbar, 2 * sizeof(unsigned), "grid barrier");
+  DG_ALLOC(m->gbar, sizeof(unsigned), "grid barrier");
   m->small_stepper = 1;
   m->Fb = Fb;
   m->n_state_faces = n_state;

@@ -197,7 +197,7 @@ struct dg_mesh {
   size_t adj_doubles;
   dg::Timing *timing;
   dg::GraphCache *graph;
-  unsigned *gbar;              // [2] grid barrier of the fused small-mesh stepper (count, generation)
+  unsigned *gbar;              // grid barrier of the fused small-mesh stepper: arrivals, cleared before each launch
   unsigned char *tc_img[2];    // B operand images of the tensor-core kernel (1xTF32, 3xTF32)
   unsigned char *split_img;    // table digits of the split-product float64 kernel; null: the mesh does not use it
   unsigned char *adj_split_img;   // the same for the adjoint's kernels; null: not used
