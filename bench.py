@@ -118,8 +118,8 @@ def _src_hash(*names) -> str:
 # voids the entry.
 TRAFFIC = {
     # k_element_split<3,4,0>, stage-2 launch (reads u^n), 256x256 p=3 vortex; then <3,4,12>
-    "1ff847c1af0f560f": 119135232 + 43563264,
-    "1ff847c1af0f560f:symmetric": 119132672 + 43329280,
+    "f824e72139886fda": 119136768 + 43352064,
+    "f824e72139886fda:symmetric": 119132928 + 43101696,
 }
 
 

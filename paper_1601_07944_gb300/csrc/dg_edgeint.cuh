@@ -5,8 +5,8 @@
  * The flux of lax_friedrichs_edge takes 54 float64 operations a point, and this
  * GPU issues 2 float64 FMAs per clock and SM, but 128 integer instructions.  Here
  * the normal velocities, the pressures, the sound speeds and the dissipation are
- * formed in fixed point (60 to 62 significant bits, so each step's error is below
- * a float64 rounding), and only the ten multiply-adds of the four results stay in
+ * formed in fixed point (60 to 62 bits relative to the largest value that the inputs'
+ * exponents allow, so each step's error is below a float64 rounding of that), and only the ten multiply-adds of the four results stay in
  * float64.
  *
  * A fixed-point number is an int64 F and an exponent X that depends on the
@@ -14,7 +14,7 @@
  * mul(a, b) = a b / 2^62, from 31-bit halves.  Both sides share the exponent of
  * the momenta, of the energies and of w, so that sums need no alignment.
  *
- * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 20 us
+ * Measured (256 x 256 mesh, one launch, float64 form -> here): k_face 47 -> 21 us
  * (p = 1), 66 -> 29 (p = 2), 87 -> 37 (p = 3), 105 -> 45 (p = 4), 124 -> 54 (p = 5);
  * k_face_mixed 88 -> 42 us (p = 3), 403 -> 173 us (512 x 512, p = 4).  Against 113-bit arithmetic the
  * error is 0.75-1.0 of the float64 form's (rms) over still, slow, supersonic and
@@ -22,7 +22,8 @@
  *
  * A point whose sides differ by more than 2^4 in density or energy, whose state is
  * not physical or not finite, whose exponents are far from one (beyond 2^300), or
- * whose (gamma - 1) P w may be below the normal range, is left to the float64 form: edge_flux_fixed returns false and writes nothing.
+ * whose (gamma - 1) P w may be below the normal range, is left to the float64 form:
+ * edge_flux_fixed returns false and writes nothing.
  */
 #pragma once
 

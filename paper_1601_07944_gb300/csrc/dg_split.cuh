@@ -29,10 +29,10 @@
  * each of GEMM 2's K steps.)
  *
  * Measured (256 x 256 mesh, 131,072 elements, one launch of a stage, k_element_sf
- * -> here): p = 1 0.108 -> 0.084 ms, p = 2 0.265 -> 0.127, p = 3 0.498 -> 0.181,
- * p = 4 0.907 -> 0.319, p = 5 1.49 -> 0.466; the symmetric rules 0.101 -> 0.081,
- * 0.242 -> 0.114, 0.593 -> 0.170, 1.08 -> 0.222, 2.07 -> 0.392; the traces alone
- * (mode 2) 0.043 -> 0.033 (p = 2), 0.074 -> 0.041 (p = 3), 0.271 -> 0.072 (p = 5).
+ * -> here): p = 1 0.108 -> 0.082 ms, p = 2 0.265 -> 0.127, p = 3 0.498 -> 0.182,
+ * p = 4 0.907 -> 0.320, p = 5 1.49 -> 0.463; the symmetric rules 0.101 -> 0.079,
+ * 0.242 -> 0.114, 0.593 -> 0.169, 1.08 -> 0.224, 2.07 -> 0.386; the traces alone
+ * (mode 2) 0.043 -> 0.032 (p = 2), 0.074 -> 0.039 (p = 3), 0.271 -> 0.074 (p = 5).
  * The float64 pipe is 60-70 % busy; the rest is the latency of a group's phases,
  * which the other groups fill only in part.  The error of the right-hand side
  * against an 80-bit reference falls by 1.5 (p = 2) to 2.9 (p = 5).
