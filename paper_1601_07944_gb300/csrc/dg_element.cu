@@ -979,14 +979,16 @@ const int *small_per_sm(int dev) {
   auto k0 = k_rk_small<P, NE, Q, kSmallTiles[0]>;
   auto k1 = k_rk_small<P, NE, Q, kSmallTiles[1]>;
   const int s0 = SmallCfg<P, NE, Q, kSmallTiles[0]>::SMEM, s1 = SmallCfg<P, NE, Q, kSmallTiles[1]>::SMEM;
-  r[0] = r[1] = 0;
+  int v[2] = {0, 0};           // (r is written once complete: two threads may ask at the same time)
   if (cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, s0) != cudaSuccess ||
       cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, s1) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r[0], k0, kSmallThreads, s0) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r[1], k1, kSmallThreads, s1) != cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v[0], k0, kSmallThreads, s0) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v[1], k1, kSmallThreads, s1) != cudaSuccess) {
     cudaGetLastError();
-    r[0] = r[1] = 0;
+    v[0] = v[1] = 0;
   }
+  r[0] = v[0];
+  r[1] = v[1];
   if (dev >= 0 && dev < 64) ready.set(dev);
   return r;
 }

@@ -167,3 +167,53 @@ def test_large_mesh_keeps_separate_launches(dgmod):
     kt = m.kernel_times()
     m.set_timing(False)
     assert "stepper" not in kt and kt["element"][0] == 6
+
+
+THREADS = r'''
+import sys, threading
+import torch
+sys.path.insert(0, ROOT)
+from paper_1601_07944_gb300 import dg, inputs as I
+dg.load()
+mesh = I.periodic_mesh(12)
+torch.zeros(1, device="cuda")
+go = threading.Barrier(8)
+made = [None] * 8
+
+def make(i):
+    torch.cuda.set_device(0)
+    go.wait()
+    made[i] = dg.Mesh.from_mesh(mesh, 2)
+
+threads = [threading.Thread(target=make, args=(i,)) for i in range(8)]
+for t in threads:
+    t.start()
+for t in threads:
+    t.join()
+first = None
+for m in made:
+    states = []
+    for fused in (True, False):
+        m.set_small_mesh_stepper(fused)
+        c = m.project_function(I.vortex)
+        m.set_timing(True)
+        m.rk_step(c, 1e-3, 3)
+        assert ("stepper" in m.kernel_times()) == fused
+        m.set_timing(False)
+        states.append(c)
+    first = states[0] if first is None else first
+    assert all(torch.equal(s, first) for s in states)
+print("threads agree")
+'''
+
+
+def test_meshes_created_by_threads_at_once():
+    """Whether a mesh fits the stepper is asked once per process, at the first mesh; eight
+    threads create theirs at once, and every one keeps the stepper and its bits."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % root + THREADS], cwd=root, capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and "threads agree" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
