@@ -298,3 +298,21 @@ def test_rows_far_from_one(dgmod, oracle_mod, p, ne, rule, k):
         u = o.project_ic(I.perturbed_vortex) + 0.002 * rng.standard_normal((o.N, 4, o.np))
         lam = rng.standard_normal(u.shape)
         assert rel_l2(_host(m.rhs_adjoint(_dev(u), _dev(lam * unit))) / unit, o.rhs_vjp(u, lam)) < 1e-12
+
+
+@pytest.mark.parametrize("p,rule", [(3, "collapsed"), (4, "collapsed"), (4, "symmetric"), (5, "collapsed"), (5, "symmetric")])
+def test_rows_lined_up_with_a_table(dgmod, oracle_mod, p, rule):
+    """Momentum rows that are a column of the interpolation or the trace table (a delta at
+    one of its points): their digits are the table's, so that the products of one level
+    all have one sign for that point."""
+    mesh = I.periodic_mesh(61)
+    m = dgmod.Mesh.from_mesh(mesh, p, vol_rule=rule)
+    o = oracle_mod.OracleDG.from_mesh(mesh, p, vol_rule=rule)
+    c = o.project_ic(_gas(0.1, 0.1, 0, 0))
+    phi = dgmod.volume_rule(p, rule)[3]
+    face = dgmod.host_tables(p)["phi_face"].reshape(-1, phi.shape[1])
+    cols = np.concatenate([phi, face])
+    for k in (1, 2):
+        c[:, k] = 1e-3 * (-1.0) ** k * cols[(np.arange(mesh.n_elem) * k) % len(cols)]
+    check_rhs(m, o, c)
+    m.device_status()
